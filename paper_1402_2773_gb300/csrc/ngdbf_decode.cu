@@ -358,7 +358,7 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     const bool state = (P->variant & 3) != 0;
     const bool adapt = (P->variant & NGDBF_ADAPT) != 0;
-    const bool wide = C->dv_max > 7;
+    const bool wide = C->dv_max > kNarrowDegree;
     PlacementChoice pc;
     ngdbf_status s = choose_placement(dev, C->n, C->m, P->t_max, C->dv_max, C->dc_max, adapt, state, smem_optin,
                                       [&](bool st) { return (const void*)pick_kernel(P->variant, P->precision, st, wide); },
@@ -394,6 +394,61 @@ float acc_scale(const ngdbf_params* P) { return (float)(std::ldexp(1.0, P->q_bit
 int32_t acc_steps(float v, float Rd) {
     const float a = v * Rd;
     return (int32_t)std::lrint(a);
+}
+
+// Margin quantization of the lazy evaluation (ngdbf_kernels.cuh) from the job's held weight,
+// thresholds and perturbation scale.  In units of y: the step is 2 w / K for a whole number K,
+// at least an eighth of the perturbation's scale (a margin is then resolved to an eighth of a
+// standard deviation: the queued outputs are about 1.7 times the flips, and a step half as
+// wide would not leave a byte room for the counts), and wide enough that the counts of a
+// symbol of the largest degree span at most kMarginCounts steps.
+void fill_margins(const ngdbf_code* C, const ngdbf_params* P, const uint32_t* thr, Job* out) {
+    Job& J = *out;
+    auto held = [&](uint32_t word) -> double {          // a threshold word in its held units
+        if (P->precision == NGDBF_FIX || P->precision == NGDBF_FIXACC) return (double)(int32_t)word;
+        float f;
+        std::memcpy(&f, &word, 4);
+        return (double)f;
+    };
+    const double scale = J.scale, d = C->dv_max;
+    double unit = 1.0, w = J.w;
+    if (P->precision == NGDBF_FIX) {
+        unit = 0.5 / (double)J.fix_R;
+        w = J.fix_W * unit;
+    } else if (P->precision == NGDBF_FIXACC) {
+        unit = 1.0 / (double)J.acc_R;
+        w = J.acc_W * unit;
+    }
+    // (a weight that quantizes to zero leaves one step per check: a lower margin, as allowed)
+    const double step0 = std::max(std::max(scale / 8.0, 2.0 * w * d / kMarginCounts), 1e-30);
+    const int K = std::max(1, (int)std::min(std::floor(2.0 * w / step0), (double)(kMarginCounts / C->dv_max)));
+    const double step = std::max(step0, 2.0 * w / K);
+    // thresholds rise towards 0 when negative; the largest one a symbol can have reached
+    const bool rising = held(thr[0]) < held(thr[P->t_max]) && (P->variant & NGDBF_ADAPT);
+    // (single-bit: the lowest guess of a slot's least E_k, below where it lies for most frames)
+    const double hi = J.single ? -1.5 * w * d / unit : rising ? held(thr[P->t_max]) : held(thr[0]);
+    // what E_k as computed may lie below its real value where it is near the threshold (beyond
+    // the byte's range the decision is monotone in the sample), in the arithmetic's roundings
+    const double ymag = J.clamp ? 1.001 * J.y_max : 300.0 * step;
+    const double mag = 2.0 * (std::fabs(hi * unit) + ymag) + 4.0 * w * d + 16.0 * scale;
+    double slack = std::ldexp(mag, -21);
+    if (P->precision == NGDBF_FP16) slack = std::ldexp(2.0 * ymag + 4.0 * w * d + 16.0 * scale, -11) + 1e-6;
+    else if (P->precision == NGDBF_FIX) slack += 1.001 * unit;
+    else if (P->precision == NGDBF_FIXACC) slack += 0.501 * unit;
+    const double round = 0.02 + std::ldexp(std::fabs((J.single ? hi : held(thr[0])) * unit) / step, -21);    // FP32 evaluation of the bytes
+    const int dcap = rising ? (int)std::min((double)(kMargin0 - K * C->dv_max), std::floor((hi - held(thr[0])) * unit / step)) : 0;
+    J.pf_inv = (float)(1.0 / step);
+    J.pf_w = (float)(w / step);
+    J.pf_bias = (float)(kMargin0 - (hi * unit + slack) / step - round);
+    J.pf_lo = (float)(K * C->dv_max);
+    J.pf_hi = (float)(255 - dcap);
+    J.pf_unit = (float)unit;
+    J.pf_d0 = rising || J.single ? (float)(hi * unit / step - round) : 0.0f;
+    J.pf_d1 = J.single ? (float)(1.0 / step) : rising ? (float)(unit / step) : 0.0f;
+    J.pf_rho = scale > 0.0 ? (float)std::min(step / scale * (1.0 - 1e-6), 1e6) : 1e6f;
+    J.pf_low = (float)(hi * unit);
+    J.pf_K = K;
+    J.pf_dcap = dcap;
 }
 
 // Job fields of one decode and its threshold words thr[0..t_max].
@@ -443,6 +498,8 @@ void fill_job(const ngdbf_code* C, const ngdbf_params* P, const float* y, int64_
         thr[u] = word;
         p = p * (double)P->lambda;
     }
+    J.slots = kSlots;
+    fill_margins(C, P, thr, &J);
 }
 
 // Kernel arguments of one decode: scratch at `base` (work counter, then the
@@ -624,14 +681,15 @@ ngdbf_status ngdbf_code_create(int32_t n, int32_t m, const int32_t* row_ptr, con
     std::vector<uint16_t> chk((size_t)dc_max * m, (uint16_t)n);
     for (int i = 0; i < m; ++i)
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) chk[(size_t)(e - row_ptr[i]) * m + i] = (uint16_t)col_idx[e];
-    // M(k) row-major [k][j], padded with the zero-word sentinel m
-    std::vector<uint16_t> sym((size_t)n * dv_max, (uint16_t)m);
+    // M(k) by groups of four symbols [k/4][j][k%4], padded with the zero-word sentinel m, so that
+    // one 8-byte load gives the j-th check of the four symbols of a group
+    std::vector<uint16_t> sym((size_t)pad4(n) * dv_max, (uint16_t)m);
     std::vector<uint8_t> deg(n);
     std::vector<int32_t> fill(n, 0);
     for (int i = 0; i < m; ++i)
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
             const int c = col_idx[e];
-            sym[(size_t)c * dv_max + fill[c]++] = (uint16_t)i;
+            sym[((size_t)(c >> 2) * dv_max + fill[c]++) * 4 + (c & 3)] = (uint16_t)i;
         }
     for (int k = 0; k < n; ++k) deg[k] = (uint8_t)sdeg[k];
 
@@ -1072,7 +1130,7 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     // shared memory for the largest code and T; state, then tables, move out when needed
     const bool state = (variant & 3) != 0, adapt = (variant & NGDBF_ADAPT) != 0;
-    T.wide = T.dv_max > 7;
+    T.wide = T.dv_max > kNarrowDegree;
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, multi_kernel_fn(variant, precision, state, T.wide));
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");

@@ -43,6 +43,35 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
+// The same function for a fixed iteration t and frame id and many groups g (counter (g, t, frame)):
+// the frame's first-round product and the second-round product of (frame, t) do not depend on
+// g and are formed once, which leaves 18 of the 20 wide multiplies per call.
+struct PhiloxLane {
+    uint32_t fhi, lo1, h0, l0;
+    __device__ __forceinline__ PhiloxLane(uint64_t frame, uint32_t t, const GenConsts& G) {
+        fhi = (uint32_t)(frame >> 32);
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint32_t)frame;
+        const uint64_t q0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ t ^ G.rk0[0]);
+        lo1 = (uint32_t)p1 ^ G.rk0[1];
+        h0 = (uint32_t)(q0 >> 32) ^ G.rk1[1];
+        l0 = (uint32_t)q0;
+    }
+    __device__ __forceinline__ void group(uint32_t g, const GenConsts& G, uint32_t out[4]) const {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * g;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(p0 >> 32) ^ fhi ^ G.rk1[0]);
+        uint32_t c0 = (uint32_t)(p1 >> 32) ^ lo1, c1 = (uint32_t)p1, c2 = h0 ^ (uint32_t)p0, c3 = l0;
+#pragma unroll
+        for (int r = 2; r < 10; ++r) {
+            const uint64_t a = (uint64_t)0xD2511F53u * c0, b = (uint64_t)0xCD9E8D57u * c2;
+            c0 = (uint32_t)(b >> 32) ^ c1 ^ G.rk0[r];
+            c2 = (uint32_t)(a >> 32) ^ c3 ^ G.rk1[r];
+            c1 = (uint32_t)b;
+            c3 = (uint32_t)a;
+        }
+        out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
+    }
+};
+
 // Standard normal deviate of one Philox output r by inversion of the normal CDF.
 // Bit 31 of r is the sign; a = 2 (r mod 2^31) + 1 gives the lower-tail probability
 // p = a 2^-33 in (0, 1/2).  With j = clz(a) and m = a << j, p lies in the j-th dyadic

@@ -11,26 +11,44 @@
 //   B. retires slots whose frame satisfied every check (pass) or reached T
 //      (smoothed output, Sec. III-E), writes their outputs, takes new frames
 //      from a global atomic queue for them and loads those frames,
-//   A'. adds, per symbol, the unsatisfied-check words of M(k) lane-wise (one
-//      4-bit lane per slot; bit-sliced for symbol degrees above 7) into the
-//      count of unsatisfied checks, shared by the 32 slots, then
-//   C. runs Step 2 / Step 3b (or Step 3a) for every symbol of every live slot:
-//      a warp processes four symbols (one Philox call) at a time with lane =
-//      slot, reads the lane's count, forms E_k = x_k y_k + w S_k + q_k, compares
-//      it with theta lambda^{u_k}, adapts u_k, accumulates the smoothing counter,
-//      and rebuilds the decision word with a warp ballot.
+//   A'. adds, per symbol, the unsatisfied-check words of M(k) lane-wise (2-bit
+//      lanes, three checks at a time, widened to 4-bit counts; bit-sliced for
+//      symbol degrees above 15) into the count of unsatisfied checks, then
+//   C. runs Step 2 / Step 3b for every symbol of every live slot: each lane draws
+//      the Philox outputs of one slot's four symbols and compares each with a cutoff
+//      that no flip can exceed (see "Lazy evaluation"); the few outputs at or below
+//      it are queued and only for those E_k = x_k y_k + w S_k + q_k is formed and
+//      compared with theta lambda^{u_k} (Step 3a: with the slot's least so far).  Symbol
+//      degrees above 15 form E_k for every symbol, with lane = slot.
 // Slots therefore iterate independently (each frame has its own t), a
 // converged frame frees its slot at once, and the CTA only stops when the
 // queue is empty and its last slot finished.
 //
-// Per-(symbol, slot) state: the held sample (global scratch, L2-resident), and a
-// 16-bit word holding u_k (bits 0-8) and the number of -1 decisions inside the
-// smoothing window (bits 9-15), in shared memory when it fits, else in global
-// scratch.  Both are laid out by groups of four symbols, [k/4][slot][k%4], so
-// that phase C reads one vector per lane for the four symbols of a Philox call;
-// the count words likewise ([k/4][slot quarter][k%4]) and the decision words
-// are contiguous.  Decision and syndrome words, counts, the threshold and
-// generator tables live in shared memory, the adjacency tables there when they fit.
+// Per-(symbol, slot) state: one byte of quantized margin (global scratch, L2-resident; the
+// dense forms hold the sample itself there), and a 16-bit word holding the flips of the symbol
+// so far (bits 0-8; u_k = t - flips) and the number of -1 decisions the smoothing window will
+// have seen at T if the symbol flips no more (bits 9-15), in shared memory when it fits, else
+// in global scratch.  Both change only when a symbol flips.  Both are laid out by groups of
+// four symbols, [k/4][slot][k%4], so that phase C reads one word per lane for the four symbols
+// of a Philox call; the counts likewise, and the decision words are contiguous.  Decision and
+// syndrome words, counts, the threshold and generator tables live in shared memory, the
+// adjacency tables there when they fit.
+//
+// Lazy evaluation.  A symbol flips only when E_k < theta_k, that is when its perturbation is
+// below -(x_k y_k + w S_k - theta_k); with z monotone in the Philox output r (r < 2^31 gives
+// the negative deviates, in increasing order) that is r below a cutoff of the margin alone.
+// Per slot the margin is kept in steps of Job::pf: a byte holds x_k y_k + w d_k - theta_hi
+// rounded down, theta_hi the largest threshold the symbol can reach; w S_k = w d_k - 2 w c
+// subtracts pf_K steps per unsatisfied check (one multiply for the four bytes of a group),
+// and the lanes of a slot at iteration t add D(t), theta_hi - theta(t) in steps rounded down
+// (theta lambda^u <= theta(t) for u <= t).  A 256-entry table maps the byte to the cutoff,
+// rounded up.  Every rounding errs towards evaluating E_k, so the decisions are those of the
+// dense form bit for bit; the exact form runs for the symbols at or below the cutoff only.
+//
+// The single-bit variant (Step 3a) needs the least E_k of a slot: it sweeps with a guess tau, the
+// slot's previous least E_k plus kGuess of its noise, in the place of the threshold.  A least
+// E_k at or below tau is the slot's (every symbol that could be as low was evaluated); the
+// slots without one are swept again with tau raised, at last with every symbol evaluated.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -56,8 +74,19 @@ constexpr int kTabChk = 1;              // N(i) table in shared memory
 constexpr int kTabSym = 2;              // M(k) table and degrees in shared memory
 
 constexpr int kMaxT = NGDBF_MAX_T;
-constexpr uint32_t kUMask = 0x1FFu;   // u_k: bits 0-8
+constexpr uint32_t kUMask = 0x1FFu;   // flips of the symbol so far: bits 0-8
 constexpr int kCShift = 9;            // smoothing count: bits 9-15
+constexpr int kNarrowDegree = 15;     // largest symbol degree of the 4-bit counts
+
+// Lazy evaluation: margin byte kMargin0 is a margin of zero (at or below it every output is
+// evaluated), pf_K d_v is at most kMarginCounts and pf_K d_v + D(t) at most kMargin0, so that
+// no byte of a group borrows from or carries into another.
+constexpr int kMargin0 = 96, kMarginCounts = 80;
+constexpr int kQueue = 32;            // outputs queued per warp for the exact form
+// Single-bit: the least E_k is guessed kGuess noise scales above the last, the first kFirst above
+// the lowest tau followed, raised by kRaise at a time and to infinity after kSweeps sweeps.
+constexpr float kGuess = 1.5f, kFirst = 2.0f, kRaise = 2.0f;
+constexpr int kSweeps = 5;
 
 // Arithmetic of the held samples and of E_k (Sec. IV-E): the perturbation is
 // always the FP32 generator output.
@@ -92,6 +121,15 @@ struct Job {
     int32_t fix_kmax, fix_W;
     float acc_R;                // FIXACC: accumulator steps per unit fl32(2^(Q+8) / Y_max), w in steps
     int32_t acc_W;
+    // lazy evaluation (see the top; real units are those of y): steps per unit, w in steps, the
+    // byte of x_k y_k + w d_k = 0, the byte's range, D(t) = floor(pf_d0 - pf_d1 theta(t)) <=
+    // pf_dcap with theta(t) as held in thr (single-bit: the shift floor(pf_d0 - pf_d1 tau) <= 0
+    // of the byte, its zero margin at the lowest tau followed), real value of one integer unit
+    // (fixed point) or 1, steps per unsatisfied check, the step in units of `scale`
+    // (rounded down), and single-bit: the lowest tau followed
+    float pf_inv, pf_w, pf_bias, pf_lo, pf_hi, pf_d0, pf_d1, pf_unit, pf_rho, pf_low;
+    int32_t pf_K, pf_dcap;
+    int32_t slots;              // frames a CTA takes first (1..32): the batch spread over the launch
     // thresholds theta lambda^u, u = 0..T: FP32 bits, binary16 values as FP32 bits, or
     // fixed-point levels Theta~(u) (FIX) or steps (FIXACC) as int32 (device memory; the
     // single-job launch passes them inline instead)
@@ -133,6 +171,7 @@ struct ChainCtx {
     int8_t* slot_e;             // [kSlots] shared memory
     int* cur_e;                 // shared memory
     Next next;
+    uint32_t* cut;              // [kChain][256] shared memory: cutoff table of each entry's job
 };
 
 // Claims up to k consecutive frames of job A: returns true and the first frame id in *base
@@ -209,16 +248,16 @@ __host__ __device__ inline Split split_range(int rank, int size, int n) {
 __host__ __device__ inline int split_local_max(int n, int size) { return 32 * (((n + 31) / 32 + size - 1) / size); }
 
 struct SmemLayout {
-    int32_t off_frame, off_start, off_ctl, off_best, off_trace, off_icdf, off_xw, off_sw, off_cnt, off_thr, off_st,
-        off_chk, off_sym, total;
+    int32_t off_frame, off_start, off_ctl, off_best, off_tau, off_trace, off_icdf, off_cut, off_queue, off_xw, off_sw, off_cnt,
+        off_thr, off_st, off_chk, off_sym, total;
 };
 
 // Offsets in bytes of the shared-memory arrays.  ctl holds: [0..1] unsatisfied
 // masks (double-buffered by pass parity), [2] live mask, [3] new-slot mask.
-// When d_v <= 7 (narrow), sw holds per check four words with one 4-bit lane per slot
-// (lane f & 7 of word f >> 3: 1 when check i is unsatisfied for slot f), and cnt holds
-// per symbol, in the same lanes, S_k + 8 = d_v(k) + 8 - 2 (unsatisfied checks in M(k)),
-// as words [k/4][quarter f >> 3][k%4] (16 bytes per symbol).  Otherwise (wide) sw holds
+// When d_v <= 15 (narrow), sw holds per check two words with one 2-bit lane per slot (lane
+// f & 15 of word f >> 4: 1 when check i is unsatisfied for slot f), and cnt holds per group of
+// four symbols sixteen words of their counts of unsatisfied checks: byte k % 4 of word
+// cnt_word(f), nibble cnt_shift(f) (16 bytes per symbol).  Otherwise (wide) sw holds
 // the 32-bit unsatisfied mask of each check and cnt, per symbol, the bit-sliced count
 // (seven words, bit f for slot f) and d_v(k) (32 bytes).  xw has room for whole groups
 // and the zero sentinel word at index n.
@@ -228,7 +267,7 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
                                                   bool need_thr, bool st_smem, int tables, int n_local = -1,
                                                   int wide = -1) {
     if (n_local < 0) n_local = n;   // symbols whose counts, state and M(k) rows this CTA holds
-    const bool wd = wide < 0 ? dv_max > 7 : wide != 0;
+    const bool wd = wide < 0 ? dv_max > kNarrowDegree : wide != 0;
     SmemLayout L;
     int o = 0;
     auto take = [&](int bytes, int align) {
@@ -242,17 +281,20 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     L.off_start = take(kSlots * 4, 16);
     L.off_ctl = take(8 * 4, 16);
     L.off_best = take(2 * kSlots * 8, 16); // single-bit variant: least (E key, k) per slot, two rounds
+    L.off_tau = take(kSlots * 4, 16);      // single-bit variant: guess of each slot's least E_k
     L.off_trace = take(kSlots * 12, 16);   // objective trace: per slot C (int64), then U (int32)
     L.off_icdf = take(256 * 16, 16);       // inverse normal CDF coefficients
+    L.off_cut = take(256 * 4, 16);         // cutoff of each margin byte
+    L.off_queue = take(32 * kQueue * 8, 16);   // per warp: outputs for the exact form
     L.off_cnt = take(pad4(n_local) * cnt_bytes, 16);
     L.off_xw = take(pad4(n + 1) * 4, 16);
-    L.off_sw = take((m + 1) * (wd ? 4 : 16), 16);
+    L.off_sw = take((m + 1) * (wd ? 4 : 8), 16);
     // all 512 values of the 9-bit u field: an idle slot's counter may pass T (its lookups are
     // don't-care but stay inside the table)
     L.off_thr = need_thr ? take((kUMask + 1) * 4, 16) : -1;
     L.off_st = st_smem ? take(pad4(n_local) * kSlots * 2, 16) : -1;
     L.off_chk = (tables & kTabChk) ? take(dc_max * m * 2, 16) : -1;
-    L.off_sym = (tables & kTabSym) ? take(n_local * dv_max * 2 + n_local, 16) : -1;
+    L.off_sym = (tables & kTabSym) ? take(pad4(n_local) * dv_max * 2 + n_local, 16) : -1;
     L.total = (o + 15) / 16 * 16;
     return L;
 }
@@ -296,11 +338,32 @@ __device__ __forceinline__ uint32_t order_key(float v) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// Bits 0..7 of b moved to bits 0, 4, ..., 28 (one bit per 4-bit lane).
-__device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
-    b = (b | (b << 12)) & 0x000F000Fu;
-    b = (b | (b << 6)) & 0x03030303u;
-    return (b | (b << 3)) & 0x11111111u;
+// Bits 0..15 of b moved to bits 0, 2, ..., 30 (one bit per 2-bit lane).
+__device__ __forceinline__ uint32_t spread_pairs(uint32_t b) {
+    b = (b | (b << 8)) & 0x00FF00FFu;
+    b = (b | (b << 4)) & 0x0F0F0F0Fu;
+    b = (b | (b << 2)) & 0x33333333u;
+    return (b | (b << 1)) & 0x55555555u;
+}
+
+// Word of a group's sixteen count words, and bit offset in each of its four bytes, that hold
+// slot f (what widening 2-bit lanes to even and odd nibbles and gathering bytes gives).
+__device__ __forceinline__ int cnt_word(int f) { return ((f >> 4) << 3) | ((f & 1) << 2) | ((f >> 2) & 3); }
+__device__ __forceinline__ int cnt_shift(int f) { return (f & 2) << 1; }
+
+// Position of the (j+1)-th set bit of mask (j < popc(mask)), by halving.
+__device__ __forceinline__ int select_bit(uint32_t mask, int j) {
+    int pos = 0;
+#pragma unroll
+    for (int w = 16; w; w >>= 1) {
+        const int c = __popc(mask & ((1u << w) - 1u));
+        if (j >= c) {
+            j -= c;
+            mask >>= w;
+            pos += w;
+        }
+    }
+    return pos;
 }
 
 // Position of the (j+1)-th set bit of mask (j < popc(mask)).
@@ -309,13 +372,97 @@ __device__ __forceinline__ int nth_set_bit(uint32_t mask, int j) {
     return __ffs(mask) - 1;
 }
 
+// The held form of a channel sample: saturated, then rounded or quantized (Sec. IV-A, IV-E).
+template <int PREC>
+__device__ __forceinline__ typename Held<PREC>::T hold(float v, const Job& A) {
+    if (A.clamp) {
+        if (v > A.y_max) v = A.y_max;
+        if (v < -A.y_max) v = -A.y_max;
+    }
+    if constexpr (PREC == kFP32) return v;
+    else if constexpr (PREC == kFP16) return __float2half_rn(v);
+    else return (int8_t)fix_code(v, A.fix_R, A.fix_kmax);
+}
+// x(0) = sign(y): whether the held sample is negative (sign(-0) = +1).
+template <int PREC>
+__device__ __forceinline__ bool held_negative(typename Held<PREC>::T h) {
+    if constexpr (PREC == kFP32) return !(h >= 0.0f);
+    else if constexpr (PREC == kFP16) return !(__half2float(h) >= 0.0f);
+    else return h < 0;
+}
+// Sample f of job A at symbol k (a serving job's samples are read past L1).
+__device__ __forceinline__ float read_sample(const Job& A, long long frame, int k) {
+    const float* p = A.y + (size_t)frame * A.n + k;
+    return A.gen ? __ldcg(p) : __ldg(p);
+}
+
+// E_k = ((x_k y_k) + w S_k) + q_k in the arithmetic of PREC, rounded after every operation
+// (Step 2): FP32 and FP16 give it as an FP32 value, the fixed-point forms as an integer.
+template <int PREC> struct Metric { using T = int32_t; };
+template <> struct Metric<kFP32> { using T = float; };
+template <> struct Metric<kFP16> { using T = float; };
+template <int PREC>
+__device__ __forceinline__ typename Metric<PREC>::T metric(typename Held<PREC>::T h, uint32_t xsign, int S, float q,
+                                                           const Job& A) {
+    if constexpr (PREC == kFP32) {
+        const float xy = __uint_as_float(__float_as_uint(h) ^ xsign);
+        return __fadd_rn(__fadd_rn(xy, __fmul_rn(A.w, __int2float_rn(S))), q);
+    } else if constexpr (PREC == kFP16) {
+        // fl(w S_k) is the exact product of a binary16 w and a small integer; the additions are
+        // binary16 additions (a correctly rounded FP32 addition of binary16 operands rounded
+        // once more to binary16 gives the same value)
+        const __half xy = __ushort_as_half(__half_as_ushort(h) ^ (uint16_t)(xsign >> 16));
+        const float ws = __fmul_rn(A.w, __int2float_rn(S));
+        return __half2float(__hadd(__hadd(xy, __float2half_rn(ws)), __float2half_rn(q)));
+    } else if constexpr (PREC == kFIX) {
+        // Eq. 9 in units of Delta/2, exact integers
+        const int32_t Y = 2 * (int32_t)h + 1;
+        const int32_t Qv = 2 * fix_code(q, A.fix_R, A.fix_kmax) + 1;
+        return (xsign ? -Y : Y) + A.fix_W * S + Qv;
+    } else {
+        // the held Eq. 8 level in accumulator steps (2^8 per half level), plus the weight and
+        // the perturbation rounded to steps: exact int32
+        const int32_t Y = (2 * (int32_t)h + 1) * (1 << kAccBits);
+        const int32_t Qs = __float2int_rn(__fmul_rn(q, A.acc_R));
+        return (xsign ? -Y : Y) + A.acc_W * S + Qs;
+    }
+}
+template <int PREC>
+__device__ __forceinline__ bool below(typename Metric<PREC>::T e, uint32_t th_bits) {
+    if constexpr (PREC == kFP32 || PREC == kFP16) return e < __uint_as_float(th_bits);
+    else return e < (int32_t)th_bits;
+}
+
+// Margin byte of a symbol of degree deg with decision sign xsign (see "Lazy evaluation"): a NaN
+// takes the low end, where every output is evaluated.
+template <int PREC>
+__device__ __forceinline__ uint32_t margin_byte(typename Held<PREC>::T h, uint32_t xsign, int deg, const Job& A) {
+    float v;
+    if constexpr (PREC == kFP32) v = h;
+    else if constexpr (PREC == kFP16) v = __half2float(h);
+    else v = (float)((2 * (int32_t)h + 1) * (PREC == kFIXACC ? (1 << kAccBits) : 1)) * A.pf_unit;
+    v = __uint_as_float(__float_as_uint(v) ^ xsign);
+    const float b = __fmaf_rn(v, A.pf_inv, __fmaf_rn(A.pf_w, (float)deg, A.pf_bias));
+    return (uint32_t)__float2int_rd(fminf(fmaxf(b, A.pf_lo), A.pf_hi));
+}
+
+// Cutoff of margin byte b: no output above it can flip a symbol whose margin is b - kMargin0 steps
+// or more.  The relative error of erfcf and of the deviates is covered by the added terms.
+__device__ __forceinline__ uint32_t margin_cutoff(int b, const Job& A) {
+    if (b <= kMargin0) return 0xFFFFFFFFu;
+    const float a = (float)(b - kMargin0) * A.pf_rho - 1e-3f;      // in units of `scale`
+    const float p = A.uniform ? 0.5f * (1.0f - a) : 0.5f * erfcf(a * 0.70710678f);
+    const float c = p * 4294967296.0f * 1.0001f + 2.0f;
+    return a <= 0.0f || c >= 4294967040.0f ? 0xFFFFFFFFu : (c > 0.0f ? (uint32_t)c : 0u);
+}
+
 // Objective trace (Sec. III-B objective f(x) = sum_k x_k y_k + sum_i s_i): for the live slots whose
 // frame id is below A.trace_frames, records at this syndrome test t the number of unsatisfied
 // checks U(t) and C(t) = sum_k rint(x_k(t) y~_k 2^32) (each term exact in double; integer sums are
 // independent of their order).  CTA-wide; every thread calls it with the same `live`.
 template <int PREC>
 __device__ __forceinline__ void trace_round(const Job& A, const SmemLayout& L, const uint16_t* chk_cols,
-                                         const typename Held<PREC>::T* ys, uint32_t live, int round) {
+                                         uint32_t live, int round) {
     extern __shared__ __align__(16) unsigned char smem[];
     const long long* lane_frame = reinterpret_cast<const long long*>(smem + L.off_frame);
     const int32_t* lane_start = reinterpret_cast<const int32_t*>(smem + L.off_start);
@@ -351,13 +498,14 @@ __device__ __forceinline__ void trace_round(const Job& A, const SmemLayout& L, c
             const int f = __ffs(r) - 1;
             long long term = 0;
             if (k < n) {
+                const typename Held<PREC>::T h = hold<PREC>(read_sample(A, lane_frame[f], k), A);
                 double v;
                 if constexpr (PREC == kFP32) {
-                    v = (double)ys[gidx(k, f)];
+                    v = (double)h;
                 } else if constexpr (PREC == kFP16) {
-                    v = (double)__half2float(ys[gidx(k, f)]);
+                    v = (double)__half2float(h);
                 } else {
-                    v = (double)(2 * (int32_t)ys[gidx(k, f)] + 1) * A.trace_yunit;
+                    v = (double)(2 * (int32_t)h + 1) * A.trace_yunit;
                 }
                 if ((xw[k] >> f) & 1u) v = -v;
                 term = __double2ll_rn(v * 4294967296.0);
@@ -404,10 +552,11 @@ __device__ __forceinline__ void load_held4(const int8_t* p, int8_t v[4]) {
 // claimed from the current entry and, when its job has none left, from other published jobs
 // with the same chain key, which ch.next copies into a free entry (one that no slot of `busy`
 // or of those just filled refers to).  Sets lane_frame (frame index within its job; -1 for a
-// slot left empty), lane_start = start and ch.slot_e for the filled slots; returns them.
+// slot left empty), lane_start = start and ch.slot_e for the filled slots; returns them, and
+// adds the entries filled to *loaded.
 template <class Next>
 __device__ uint32_t fill_chained(ChainCtx<Next>& ch, unsigned long long key, uint32_t want, uint32_t busy,
-                                 int start, long long* lane_frame, int32_t* lane_start) {
+                                 int start, long long* lane_frame, int32_t* lane_start, uint32_t* loaded) {
     uint32_t fresh = 0;
     for (int step = 0; step <= kChain; ++step) {
         const uint32_t left = want & ~fresh;
@@ -438,6 +587,7 @@ __device__ uint32_t fill_chained(ChainCtx<Next>& ch, unsigned long long key, uin
             if (!used) e2 = e;
         }
         if (e2 < 0 || !ch.next(key, ch.jl[e2])) break;
+        *loaded |= 1u << e2;            // its cutoff table is made at the refill
         *ch.cur_e = e2;
     }
     for (uint32_t r = want & ~fresh; r; r &= r - 1) lane_frame[__ffs(r) - 1] = -1;
@@ -463,7 +613,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                                            const SmemLayout& L, int tables,
                                            typename Held<PREC>::T* ys, uint16_t* st_cta,
                                            Split S = Split{0, 1, 0, 0},
-                                           ChainCtx<Next> ch = ChainCtx<Next>{nullptr, nullptr, nullptr, Next{}}) {
+                                           ChainCtx<Next> ch = ChainCtx<Next>{nullptr, nullptr, nullptr, Next{}, nullptr}) {
     static_assert(!(CL && CHAIN), "chained jobs are not split over clusters");
     constexpr bool kState = ADAPT || SMOOTH;
     // the job whose frame slot f holds (per-request fields: samples, sigma, frame offset,
@@ -498,6 +648,12 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     uint32_t* sw = reinterpret_cast<uint32_t*>(smem + L.off_sw);
     unsigned long long* best = reinterpret_cast<unsigned long long*>(smem + L.off_best);
     float4* icdf = reinterpret_cast<float4*>(smem + L.off_icdf);
+    uint32_t* cut = CHAIN ? ch.cut : reinterpret_cast<uint32_t*>(smem + L.off_cut);
+    float* tau = reinterpret_cast<float*>(smem + L.off_tau);
+    const bool single = !ADAPT && A.single;
+    // wide: every symbol evaluated, with its held sample in `ys`; else margin bytes there
+    constexpr bool dense = WIDE;
+    uint8_t* yb = reinterpret_cast<uint8_t*>(ys);
     uint32_t* thr = ADAPT ? reinterpret_cast<uint32_t*>(smem + L.off_thr) : nullptr;
     uint16_t* st = nullptr;
     if constexpr (kState) {
@@ -517,8 +673,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     int sym_base = 0;           // first symbol of the M(k) rows sym_chks points to
     if (tables & kTabSym) {
         uint16_t* s = reinterpret_cast<uint16_t*>(smem + L.off_sym);
-        uint8_t* d = reinterpret_cast<uint8_t*>(s + nl * dv_max);
-        for (int i = tid; i < nl * dv_max; i += blockDim.x) s[i] = A.sym_chks[k_lo * dv_max + i];
+        uint8_t* d = reinterpret_cast<uint8_t*>(s + pad4(nl) * dv_max);
+        for (int i = tid; i < pad4(nl) * dv_max; i += blockDim.x) s[i] = A.sym_chks[k_lo * dv_max + i];
         for (int i = tid; i < nl; i += blockDim.x) d[i] = A.sym_deg[k_lo + i];
         sym_chks = s;
         sym_deg = d;
@@ -534,14 +690,14 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if constexpr (CHAIN) {
             *ch.cur_e = 0;
             for (int f = 0; f < kSlots; ++f) ch.slot_e[f] = 0;     // every slot names a loaded entry
-            live = fill_chained(ch, A.chain_key, 0xFFFFFFFFu, 0u, 0, lane_frame, lane_start);
+            live = fill_chained(ch, A.chain_key, 0xFFFFFFFFu, 0u, 0, lane_frame, lane_start, ctl + 4);
         } else {
             unsigned long long base = 0;
-            const bool got = claim_frames(A, kSlots, &base);
+            const bool got = claim_frames(A, (unsigned)A.slots, &base);
             for (int f = 0; f < kSlots; ++f) {
                 const unsigned long long fid = base + f;
                 lane_start[f] = 0;
-                if (got && fid < (unsigned long long)A.n_frames) {
+                if (got && f < A.slots && fid < (unsigned long long)A.n_frames) {
                     lane_frame[f] = (long long)fid;
                     live |= 1u << f;
                 } else {
@@ -560,7 +716,13 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     }
     for (int i = tid; i < 256; i += blockDim.x) icdf[i] = G.icdf[i];
     for (int k = tid; k < pad4(n + 1); k += blockDim.x) xw[k] = 0u;
-    for (int i = tid; i < (m + 1) * (WIDE ? 1 : 4); i += blockDim.x) sw[i] = 0u;
+    for (int i = tid; i < (m + 1) * (WIDE ? 1 : 2); i += blockDim.x) sw[i] = 0u;
+    // (an unsplit chaining CTA makes entry 0's table here, the others' when they are loaded)
+    for (int i = tid; i < 256; i += blockDim.x) cut[i] = margin_cutoff(i, A);
+    // the missing symbols of a partial last group: margins that nothing undercuts
+    if (!dense)
+        for (int e = nl * kSlots + tid; e < pad4(nl) * kSlots; e += blockDim.x)
+            yb[gidx(e / kSlots, e % kSlots)] = (uint8_t)(int)A.pf_hi;
     // a serving job's thresholds and samples were copied in while the kernel runs: read them
     // past L1, which may still hold lines of an earlier request at the same addresses
     if constexpr (ADAPT)
@@ -600,36 +762,42 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     for (;;) {
         if (refill) {
             // ---- load new frames: saturated samples into the slot columns, x(0) = sign(y) ----
+            // (four samples in flight per thread)
             const uint32_t fresh = ctl[3];
+            if (single && tid < kSlots && ((fresh >> tid) & 1u)) tau[tid] = A.pf_low + kFirst * job_of(tid).scale;
+            if constexpr (CHAIN) {
+                for (uint32_t r = ctl[4]; r; r &= r - 1) {
+                    const int e = __ffs(r) - 1;
+                    for (int i = tid; i < 256; i += blockDim.x) cut[256 * e + i] = margin_cutoff(i, ch.jl[e]);
+                }
+            }
             for (int k = k_lo + tid; k < k_hi; k += blockDim.x) {
                 uint32_t word = xw[k] & ~fresh;
-                uint32_t rest = fresh;
-                while (rest) {
-                    const int f = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    const Job& Jf = job_of(f);
-                    const float* yp = Jf.y + (size_t)lane_frame[f] * n + k;
-                    float v = Jf.gen ? __ldcg(yp) : __ldg(yp);
-                    if (A.clamp) {
-                        if (v > A.y_max) v = A.y_max;
-                        if (v < -A.y_max) v = -A.y_max;
+                const int deg = sym_deg[k - sym_base];
+                for (uint32_t rest = fresh; rest;) {
+                    int fs[4];
+                    float v[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        fs[i] = __ffs(rest) - 1;            // -1 when none is left
+                        rest &= rest - 1;
+                        v[i] = fs[i] >= 0 ? read_sample(job_of(fs[i]), lane_frame[fs[i]], k) : 0.0f;
                     }
-                    bool negative;
-                    const int at = gidx(k - k_lo, f);
-                    if constexpr (PREC == kFP32) {
-                        ys[at] = v;
-                        negative = !(v >= 0.0f);
-                    } else if constexpr (PREC == kFP16) {
-                        const __half h = __float2half_rn(v);
-                        ys[at] = h;
-                        negative = !(__half2float(h) >= 0.0f);        // sign(-0) = +1
-                    } else {
-                        const int32_t b = fix_code(v, A.fix_R, A.fix_kmax);
-                        ys[at] = (int8_t)b;
-                        negative = b < 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int f = fs[i];
+                        if (f < 0) break;
+                        const Job& Jf = job_of(f);
+                        const HeldT h = hold<PREC>(v[i], Jf);
+                        const bool negative = held_negative<PREC>(h);
+                        const int at = gidx(k - k_lo, f);
+                        if (dense) ys[at] = h;
+                        else yb[at] = (uint8_t)margin_byte<PREC>(h, negative ? 0x80000000u : 0u, deg, Jf);
+                        if (negative) word |= 1u << f;
+                        // no flips yet; without any, every x(t) of the window is x(0)
+                        if constexpr (kState)
+                            st[at] = (SMOOTH && negative) ? (uint16_t)((T - A.t_smooth + 1) << kCShift) : 0;
                     }
-                    if (negative) word |= 1u << f;
-                    if constexpr (kState) st[at] = 0;
                 }
                 xw[k] = word;
                 if constexpr (CL) {
@@ -638,6 +806,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 }
             }
             group_sync();
+            if (CHAIN && tid == 0) ctl[4] = 0u;
             refill = false;
         }
 
@@ -657,8 +826,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 if constexpr (WIDE) {
                     if (i < m && sub == 0) sw[i] = s;
                 } else {
-                    // byte `sub` of the word, one slot per 4-bit lane (slots 8 sub .. 8 sub + 7)
-                    if (i < m) sw[4 * i + sub] = spread_nibbles((s >> (8 * sub)) & 0xFFu);
+                    // half `sub` of the word, one slot per 2-bit lane (slots 16 sub .. 16 sub + 15)
+                    if (i < m && sub < 2) sw[2 * i + sub] = spread_pairs((s >> (16 * sub)) & 0xFFFFu);
                 }
                 acc |= s;
             }
@@ -670,7 +839,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         ++pass_id;
         uint32_t live = ctl[2];
         if (A.trace_u != nullptr)
-            trace_round<PREC>(A, L, chk_cols, ys, live, round);
+            trace_round<PREC>(A, L, chk_cols, live, round);
         const uint32_t conv = live & ~unsat;
         const int my_t = round - lane_start[lane];
         const uint32_t at_T = __ballot_sync(0xFFFFFFFFu, ((live >> lane) & 1u) && my_t >= T);
@@ -694,9 +863,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                         uint32_t bit = (xw[k] >> f) & 1u;
                         if constexpr (SMOOTH) {
                             if (!ok) {
-                                // X_k = terms - 2 * (#-1 decisions), x(T) included here
+                                // X_k = terms - 2 * (#-1 decisions in t_smooth .. T)
                                 const int terms = tf - A.t_smooth + 1;
-                                const int neg = (int)(st[gidx(k - k_lo, f)] >> kCShift) + (int)bit;
+                                const int neg = (int)(st[gidx(k - k_lo, f)] >> kCShift);
                                 const int X = terms - 2 * neg;
                                 bit = X < 0 ? 1u : (X > 0 ? 0u : bit);
                             }
@@ -743,7 +912,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (tid == 0 && (!split || S.rank == 0)) {
                 uint32_t fresh = 0;
                 if constexpr (CHAIN) {
-                    fresh = fill_chained(ch, A.chain_key, fin, live & ~fin, round, lane_frame, lane_start);
+                    fresh = fill_chained(ch, A.chain_key, fin, live & ~fin, round, lane_frame, lane_start, ctl + 4);
                 } else {
                     unsigned long long base = 0;
                     const bool got = claim_frames(A, (unsigned)nfin, &base);
@@ -787,28 +956,54 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if (live == 0) break;
 
         // ---- A'. per symbol and slot, the count of unsatisfied checks in M(k) ----
-        for (int k = k_lo + tid; k < k_hi; k += blockDim.x) {
-            const int kk = k - k_lo;                      // local index of the symbol
-            const uint16_t* row = sym_chks + (k - sym_base) * dv_max;
-            if constexpr (!WIDE) {
-                // d_v <= 7: one 4-bit lane per slot, counts added lane-wise without carries;
-                // stored as S_k + 8 = d_v + 8 - 2 count in [1, 15]
-                const uint4* sw4 = reinterpret_cast<const uint4*>(sw);
-                uint4 c = make_uint4(0u, 0u, 0u, 0u);
-                for (int e = 0; e < dv_max; ++e) {
-                    const uint4 s = sw4[row[e]];
-                    c.x += s.x; c.y += s.y; c.z += s.z; c.w += s.w;
+        const int groups_l = (nl + 3) >> 2;          // groups of four symbols (the code's last can be partial)
+        // a CTA of a split job flips decisions in every copy during phase C: none before every
+        // CTA has formed its syndromes (the barrier's wait is below, after the counts)
+        if constexpr (CL) {
+            if (split) cooperative_groups::this_cluster().barrier_arrive();
+        }
+        if constexpr (!WIDE) {
+            // two threads per group, each for 16 slots: the four symbols' check words added in
+            // 2-bit lanes three at a time, widened to nibbles (even and odd slots), and the
+            // bytes of the four symbols gathered into the words that phase C reads
+            const uint2* rows = reinterpret_cast<const uint2*>(sym_chks) + (size_t)((k_lo - sym_base) >> 2) * dv_max;
+            for (int i = tid; i < 2 * groups_l; i += blockDim.x) {
+                const int gl = i >> 1, h = i & 1;
+                const uint2* row = rows + (size_t)gl * dv_max;
+                uint32_t ev[4] = {0u, 0u, 0u, 0u}, od[4] = {0u, 0u, 0u, 0u};
+                for (int e = 0; e < dv_max; e += 3) {
+                    uint32_t a[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        if (e + d >= dv_max) break;
+                        const uint2 c = row[e + d];         // the d-th check of each of the four symbols
+                        a[0] += sw[2 * (c.x & 0xFFFFu) + h];
+                        a[1] += sw[2 * (c.x >> 16) + h];
+                        a[2] += sw[2 * (c.y & 0xFFFFu) + h];
+                        a[3] += sw[2 * (c.y >> 16) + h];
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        ev[j] += a[j] & 0x33333333u;
+                        od[j] += (a[j] >> 2) & 0x33333333u;
+                    }
                 }
-                const uint32_t D = ((uint32_t)sym_deg[k - sym_base] + 8u) * 0x11111111u;
-                uint32_t* cw = reinterpret_cast<uint32_t*>(cnt) + ((kk >> 2) << 4) + (kk & 3);
-                cw[0] = D - 2u * c.x;     // quarter q of the group at word 4 q + k % 4
-                cw[4] = D - 2u * c.y;
-                cw[8] = D - 2u * c.z;
-                cw[12] = D - 2u * c.w;
-            } else {
+                auto bytes = [](const uint32_t w[4]) {      // word b: byte b of w[0..3]
+                    const uint32_t t0 = __byte_perm(w[0], w[1], 0x5140), t1 = __byte_perm(w[0], w[1], 0x7362);
+                    const uint32_t u0 = __byte_perm(w[2], w[3], 0x5140), u1 = __byte_perm(w[2], w[3], 0x7362);
+                    return make_uint4(__byte_perm(t0, u0, 0x5410), __byte_perm(t0, u0, 0x7632),
+                                      __byte_perm(t1, u1, 0x5410), __byte_perm(t1, u1, 0x7632));
+                };
+                cnt[4 * gl + 2 * h] = bytes(ev);
+                cnt[4 * gl + 2 * h + 1] = bytes(od);
+            }
+        } else {
+            for (int k = k_lo + tid; k < k_hi; k += blockDim.x) {
+                const int kk = k - k_lo;                      // local index of the symbol
+                const uint16_t* row = sym_chks + ((k - sym_base) >> 2) * 4 * dv_max + (k & 3);
                 uint32_t b[7] = {0, 0, 0, 0, 0, 0, 0};     // count <= 127: seven slices
                 for (int e = 0; e < dv_max; ++e) {
-                    uint32_t carry = sw[row[e]];
+                    uint32_t carry = sw[row[4 * e]];
 #pragma unroll
                     for (int q = 0; q < 7; ++q) {
                         const uint32_t c = b[q] & carry;
@@ -820,169 +1015,201 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 cnt[2 * kk + 1] = make_uint4(b[4], b[5], b[6], (uint32_t)sym_deg[k - sym_base]);
             }
         }
+        if constexpr (CL) {
+            if (split) cooperative_groups::this_cluster().barrier_wait();
+        }
         __syncthreads();
 
+        // threshold of the non-adaptive variants
+        const uint32_t th0 = CHAIN ? th0_once : (A.gen ? __ldcg(thr_src) : thr_src[0]);
+        const int g_lo = k_lo >> 2;              // first group of this CTA's symbols
+        const uint32_t* cntw = reinterpret_cast<const uint32_t*>(cnt);
+        const bool uniform = A.uniform != 0;
+
+        // A flip of (symbol kl of this CTA, slot f) at the slot's iteration t: the flip count, and
+        // the window count, which takes the new decision for x(t + 1) .. x(T)
+        auto flipped_state = [&](uint32_t s0, bool was_neg, int t) -> uint32_t {
+            uint32_t s1 = s0 + (ADAPT ? 1u : 0u);
+            if constexpr (SMOOTH) {
+                const uint32_t rem = (uint32_t)(T - max(t + 1, A.t_smooth) + 1) << kCShift;
+                s1 = was_neg ? s1 - rem : s1 + rem;
+            }
+            return s1;
+        };
+
+        // E_k as an order-preserving key and, from the key, in real units (single-bit variant)
+        auto key_of = [](typename Metric<PREC>::T E) -> uint32_t {
+            if constexpr (PREC == kFP32 || PREC == kFP16) return order_key(E);
+            else return (uint32_t)E ^ 0x80000000u;
+        };
+        auto value_of = [&](uint32_t key) -> float {
+            if constexpr (PREC == kFP32 || PREC == kFP16)
+                return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+            else return __fmul_rn((float)(int32_t)(key ^ 0x80000000u), A.pf_unit);
+        };
+        // single-bit variant: least (E key, k) of each slot over this CTA's symbols; when split, in
+        // the buffer of this round's parity (the CTAs of the cluster read each other's)
+        unsigned long long* bcur = best + (split ? (round & 1) * kSlots : 0);
+        uint32_t todo = live;           // single-bit variant: slots whose flip is not decided yet
+
         // ---- C. Step 2 and Step 3b for every symbol of every live slot ----
-        {
+        for (int sweep = 1;; ++sweep) {
+        if constexpr (!dense) {
+            // lanes over (group, slot): `per` groups at a time when few slots are live
+            const int n_live = __popc(todo);
+            const int lg = n_live > 1 ? 32 - __clz(n_live - 1) : 0, per = 32 >> lg;
+            const int li = lane & ((1 << lg) - 1);
+            const bool act = li < n_live;
+            const int slot = n_live == 32 ? lane : select_bit(todo, act ? li : 0);
+            const Job& Jl = job_of(slot);
+            const int t = round - lane_start[slot];
+            const PhiloxLane ph(Jl.frame_offset + (uint64_t)lane_frame[slot], (uint32_t)t, G);
+            uint32_t K = (uint32_t)Jl.pf_K, D = 0u, ebase = 0u;
+            [[maybe_unused]] int shift = 0;
+            if constexpr (ADAPT) {
+                const float th = (PREC == kFP32 || PREC == kFP16) ? __uint_as_float(thr[t]) : (float)(int32_t)thr[t];
+                const float d = __fmaf_rn(-Jl.pf_d1, th, Jl.pf_d0);
+                D = (uint32_t)min((int)fminf(fmaxf(d, 0.0f), 255.0f), Jl.pf_dcap) * 0x01010101u;
+            } else if (single) {
+                shift = __float2int_rd(fminf(fmaxf(__fmaf_rn(-Jl.pf_d1, tau[slot], Jl.pf_d0), -255.0f), 0.0f));
+            }
+            if constexpr (CHAIN) ebase = (uint32_t)ch.slot_e[slot];
+            const uint32_t csh = (uint32_t)cnt_shift(slot);
+            const uint32_t* yrow = reinterpret_cast<const uint32_t*>(yb) + slot;
+            const uint32_t* crow = cntw + cnt_word(slot);
+            uint2* queue = reinterpret_cast<uint2*>(smem + L.off_queue) + warp * kQueue;
+            int queued = 0;
+
+            // the exact form for the queued outputs, one per lane
+            auto evaluate = [&](int count) {
+                __syncwarp();
+                if (lane < count) {
+                    const uint2 q = queue[lane];
+                    const int kl = (int)(q.y & 0xFFFFu), f = (int)(q.y >> 16), k = k_lo + kl;
+                    if (k < k_hi) {
+                        const Job& Jf = job_of(f);
+                        const HeldT h = hold<PREC>(read_sample(Jf, lane_frame[f], k), Jf);
+                        const int tf = round - lane_start[f];
+                        const int deg = sym_deg[k - sym_base];
+                        const uint32_t c = (cntw[(kl >> 2) * 16 + cnt_word(f)] >> (8 * (kl & 3) + cnt_shift(f))) & 0xFu;
+                        uint32_t* xk = xw + k;
+                        const uint32_t xsign = ((*(volatile uint32_t*)xk >> f) & 1u) << 31;
+                        const float z = uniform ? uniform_dev(q.x) : gauss_icdf(q.x, icdf);
+                        const auto E = metric<PREC>(h, xsign, deg - 2 * (int)c, __fmul_rn(Jf.scale, z), A);
+                        if (single) {
+                            // Step 3a: the slot's least E_k (the lowest k among equal values)
+                            const unsigned long long cand = ((unsigned long long)key_of(E) << 32) | (uint32_t)k;
+                            if (cand < *(volatile unsigned long long*)(bcur + f)) atomicMin(bcur + f, cand);
+                        } else {
+                            const int at = gidx(kl, f);
+                            [[maybe_unused]] uint32_t s0 = 0u;
+                            if constexpr (kState) s0 = st[at];
+                            if (below<PREC>(E, ADAPT ? thr[(tf - (int)(s0 & kUMask)) & kUMask] : th0)) {
+                                atomicXor(xk, 1u << f);
+                                if constexpr (CL) {
+                                    for (int r = 0; split && r < S.size; ++r)
+                                        if (r != S.rank) atomicXor(peer(xw, r) + k, 1u << f);
+                                }
+                                if constexpr (kState) st[at] = (uint16_t)flipped_state(s0, xsign != 0u, tf);
+                                yb[at] = (uint8_t)margin_byte<PREC>(h, xsign ^ 0x80000000u, deg, Jf);
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+            };
+
+            for (int g0 = warp * per; g0 < groups_l; g0 += nwarps * per) {
+                const int gl = g0 + (lane >> lg);
+                const bool ok = act && gl < groups_l;
+                const int gs = ok ? gl : 0;
+                // the loads before the generator's arithmetic, so that their latency overlaps it
+                const uint32_t y4 = yrow[gs * kSlots], c4 = crow[gs * 16];
+                uint32_t r[4];
+                ph.group((uint32_t)(g_lo + gs), G, r);
+                const uint32_t m4 = y4 + D - K * ((c4 >> csh) & 0x0F0F0F0Fu);
+                bool low[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    uint32_t i = __byte_perm(m4, ebase, 0x5540 + j);
+                    if (single) i = (i & ~0xFFu) | (uint32_t)max((int)(i & 0xFFu) + shift, 0);
+                    low[j] = r[j] <= cut[i];
+                }
+                if (__any_sync(0xFFFFFFFFu, ok && (low[0] || low[1] || low[2] || low[3]))) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool mine = ok && low[j];
+                        const uint32_t b = __ballot_sync(0xFFFFFFFFu, mine);
+                        if (b == 0u) continue;
+                        const int more = __popc(b);
+                        if (queued + more > kQueue) {
+                            evaluate(queued);
+                            queued = 0;
+                        }
+                        if (mine)
+                            queue[queued + __popc(b & ((1u << lane) - 1u))] =
+                                make_uint2(r[j], (uint32_t)(4 * gl + j) | ((uint32_t)slot << 16));
+                        queued += more;
+                    }
+                }
+            }
+            if (queued) evaluate(queued);
+        } else {
+            // every symbol of every slot, lane = slot (an idle slot's decisions and counters are
+            // don't-care: cleared when it takes a frame, never part of an output)
             const bool act = (live >> lane) & 1u;
             const long long fr = lane_frame[lane];
-            const Job& Jl = job_of(lane);           // an idle lane's entry is stale: don't-care
+            const Job& Jl = job_of(lane);
             const uint64_t fid = Jl.frame_offset + (uint64_t)(act ? fr : 0);
             const uint32_t flo = (uint32_t)fid, fhi = (uint32_t)(fid >> 32);
             const int t = act ? round - lane_start[lane] : 0;
-            const bool window = SMOOTH && act && t >= A.t_smooth;
-            const int g_lo = k_lo >> 2;              // first group of this CTA's symbols
-            // threshold of the non-adaptive variants
-            const uint32_t th0 = CHAIN ? th0_once : (A.gen ? __ldcg(thr_src) : thr_src[0]);
-            const float scale = Jl.scale, wgt = A.w, fix_R = A.fix_R, acc_R = A.acc_R;
-            const int32_t fix_kmax = A.fix_kmax, fix_W = A.fix_W, acc_W = A.acc_W;
-            const bool uniform = A.uniform != 0;
-            const bool single = !ADAPT && A.single;
-            const uint32_t nib_shift = 4u * (lane & 7);
-            const float wgt_m8 = -8.0f * wgt;       // exact
+            const float scale = Jl.scale;
             unsigned long long my_best = ~0ull;      // single-bit variant: (E key << 32) | k
-            // one group of four symbols; only the last group of a code with n % 4 != 0 is partial
-            // (its missing symbols read the zeroed padding and are skipped)
-            auto group = [&](const int gl, auto partial_tag) {
-                constexpr bool kPartial = decltype(partial_tag)::value;
-                const int g = g_lo + gl;                  // group index in the code (Philox counter)
-                const int k0 = 4 * g;
+            for (int gl = warp; gl < groups_l; gl += nwarps) {
+                const int g = g_lo + gl, k0 = 4 * g;     // group index in the code (Philox counter)
                 const int at = (gl * kSlots + lane) * 4;  // this lane's entries in the group layout
-                // issue the sample, state, count, decision-word and threshold loads (one vector
-                // each) before the generator's arithmetic, so that their latency overlaps it
                 HeldT yv[4];
                 load_held4(ys + at, yv);
-                [[maybe_unused]] uint32_t sv[4], cwv[4], thv[4];
+                [[maybe_unused]] uint32_t sv[4] = {0u, 0u, 0u, 0u}, c4 = 0u;
                 if constexpr (kState) {
                     const uint2 s2 = *reinterpret_cast<const uint2*>(st + at);
                     sv[0] = s2.x & 0xFFFFu; sv[1] = s2.x >> 16; sv[2] = s2.y & 0xFFFFu; sv[3] = s2.y >> 16;
                 }
-                if constexpr (!WIDE) {
-                    const uint4 c4 = reinterpret_cast<const uint4*>(cnt)[gl * 4 + (lane >> 3)];
-                    cwv[0] = c4.x; cwv[1] = c4.y; cwv[2] = c4.z; cwv[3] = c4.w;
-                }
+                if constexpr (!WIDE) c4 = cntw[16 * gl + cnt_word(lane)] >> cnt_shift(lane);
                 const uint4 x4 = reinterpret_cast<const uint4*>(xw)[g];
                 const uint32_t xwv[4] = {x4.x, x4.y, x4.z, x4.w};
-                if constexpr (ADAPT) {
-                    // u_k <= t - 1 < T for a live slot (cleared on every refill)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) thv[j] = thr[sv[j] & kUMask];
-                }
                 float z[4];
                 noise4((uint32_t)g, (uint32_t)t, flo, fhi, G, icdf, uniform, z);
                 uint32_t fmv[4] = {0u, 0u, 0u, 0u};          // flip masks of the four symbols
-                [[maybe_unused]] uint32_t nvv[4];             // new state words
-                if constexpr (kState) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) nvv[j] = sv[j];
-                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int k = k0 + j;
-                    if (kPartial && k >= n) break;
-                    int S;
-                    float ws;           // fl(w S_k)
+                    if (k >= k_hi) break;
+                    int Sk;
                     if constexpr (!WIDE) {
-                        // this slot's 4-bit lane of the symbol's count word: S_k + 8, and
-                        // w S_k = fl(w (S_k + 8) - 8 w) in one rounding (8 w is exact)
-                        const uint32_t nib = (cwv[j] >> nib_shift) & 0xFu;
-                        S = (int)nib - 8;
-                        ws = __fmaf_rn(wgt, __uint2float_rn(nib), wgt_m8);
+                        Sk = (int)sym_deg[k - sym_base] - 2 * (int)((c4 >> (8 * j)) & 0xFu);
                     } else {
                         const uint4 c = cnt[2 * (k - k_lo)], d = cnt[2 * (k - k_lo) + 1];
                         const int unsat_cnt = (int)(((c.x >> lane) & 1u) | (((c.y >> lane) & 1u) << 1) |
                                                     (((c.z >> lane) & 1u) << 2) | (((c.w >> lane) & 1u) << 3) |
                                                     (((d.x >> lane) & 1u) << 4) | (((d.y >> lane) & 1u) << 5) |
                                                     (((d.z >> lane) & 1u) << 6));
-                        S = (int)d.w - 2 * unsat_cnt;
-                        ws = __fmul_rn(wgt, __int2float_rn(S));
+                        Sk = (int)d.w - 2 * unsat_cnt;
                     }
-                    const uint32_t xword = xwv[j];
-                    // x_k = -1 as the sign bit of x_k y_k, and as a bool
-                    const uint32_t xsign = (xword << (31 - lane)) & 0x80000000u;
-                    [[maybe_unused]] const bool xneg = xsign != 0u;
-                    const float q = __fmul_rn(scale, z[j]);
-                    // E_k = ((x_k y_k) + w S_k) + q_k, rounded after every operation (Step 2)
-                    auto metric32 = [&]() -> float {
-                        const float xy = __uint_as_float(__float_as_uint((float)yv[j]) ^ xsign);
-                        return __fadd_rn(__fadd_rn(xy, ws), q);
-                    };
-                    // the same in binary16: each result rounded to binary16.  fl(w S_k) is the
-                    // exact product of a binary16 w and a small integer; the additions are
-                    // binary16 additions (a correctly rounded FP32 addition of binary16
-                    // operands rounded once more to binary16 gives the same value)
-                    [[maybe_unused]] auto metric16 = [&]() -> __half {
-                        if constexpr (PREC == kFP16) {
-                            const __half xy = __ushort_as_half(__half_as_ushort(yv[j]) ^ (uint16_t)(xsign >> 16));
-                            return __hadd(__hadd(xy, __float2half_rn(ws)), __float2half_rn(q));
-                        } else {
-                            return __float2half_rn(0.0f);
-                        }
-                    };
-                    // the held Eq. 8 level in accumulator steps (2^8 per half level), plus the
-                    // weight and the perturbation rounded to steps: exact int32
-                    [[maybe_unused]] auto metric_acc = [&]() -> int32_t {
-                        const int32_t Y = (2 * (int32_t)yv[j] + 1) * (1 << kAccBits);
-                        const int32_t Qs = __float2int_rn(__fmul_rn(q, acc_R));
-                        return (xneg ? -Y : Y) + acc_W * S + Qs;
-                    };
-                    // below_threshold(u): E_k < theta_k in the held arithmetic
-                    auto below = [&](uint32_t th_bits) -> bool {
-                        if constexpr (PREC == kFP32) {
-                            return metric32() < __uint_as_float(th_bits);
-                        } else if constexpr (PREC == kFP16) {
-                            return __half2float(metric16()) < __uint_as_float(th_bits);
-                        } else if constexpr (PREC == kFIX) {
-                            // Eq. 9 in units of Delta/2, exact integers
-                            const int32_t Y = 2 * (int32_t)yv[j] + 1;
-                            const int32_t Qv = 2 * fix_code(q, fix_R, fix_kmax) + 1;
-                            return (xneg ? -Y : Y) + fix_W * S + Qv < (int32_t)th_bits;
-                        } else {
-                            return metric_acc() < (int32_t)th_bits;
-                        }
-                    };
-                    if constexpr (!ADAPT) {
-                        if (single) {
-                            // Step 3a: remember this lane's least E_k; flips wait for all symbols
-                            uint32_t key;
-                            if constexpr (PREC == kFP32) {
-                                key = order_key(metric32());
-                            } else if constexpr (PREC == kFP16) {
-                                key = order_key(__half2float(metric16()));
-                            } else if constexpr (PREC == kFIXACC) {
-                                key = (uint32_t)metric_acc() ^ 0x80000000u;
-                            } else {
-                                const int32_t Y = 2 * (int32_t)yv[j] + 1;
-                                const int32_t Qv = 2 * fix_code(q, fix_R, fix_kmax) + 1;
-                                key = (uint32_t)((xneg ? -Y : Y) + fix_W * S + Qv) ^ 0x80000000u;
-                            }
-                            const unsigned long long cand = ((unsigned long long)key << 32) | (uint32_t)k;
-                            my_best = cand < my_best ? cand : my_best;
-                            if constexpr (SMOOTH) {
-                                if (window && xneg) nvv[j] = sv[j] + (1u << kCShift);
-                            }
-                            continue;
-                        }
-                    }
-                    bool flip;
-                    if constexpr (kState) {
-                        const uint32_t s0 = sv[j];
-                        const uint32_t th = ADAPT ? thv[j] : th0;
-                        const bool lower = below(th);       // evaluated for every lane, no branch
-                        // an idle slot (no frame) may flip and count too: its decision bits and
-                        // counters are cleared when it takes a frame and never reach an output
-                        flip = lower;
-                        // u_k += 1 when not flipped; the window counter counts x_k = -1
-                        nvv[j] = s0 + ((ADAPT && !flip) ? 1u : 0u) + (window ? (xsign >> (31 - kCShift)) : 0u);
+                    const uint32_t xsign = (xwv[j] << (31 - lane)) & 0x80000000u;
+                    const auto E = metric<PREC>(yv[j], xsign, Sk, __fmul_rn(scale, z[j]), A);
+                    if (single) {
+                        // Step 3a: remember this lane's least E_k; flips wait for all symbols
+                        const unsigned long long cand = ((unsigned long long)key_of(E) << 32) | (uint32_t)k;
+                        my_best = cand < my_best ? cand : my_best;
                     } else {
-                        flip = below(th0);              // idle slots: don't-care, as above
+                        const uint32_t th = ADAPT ? thr[(t - (int)(sv[j] & kUMask)) & kUMask] : th0;
+                        const bool flip = below<PREC>(E, th);
+                        if constexpr (kState) {
+                            if (flip) st[at + j] = (uint16_t)flipped_state(sv[j], xsign != 0u, t);
+                        }
+                        fmv[j] = __ballot_sync(0xFFFFFFFFu, flip);
                     }
-                    fmv[j] = __ballot_sync(0xFFFFFFFFu, flip);
-                }
-                if constexpr (kState) {
-                    const uint2 n2 = make_uint2(nvv[0] | (nvv[1] << 16), nvv[2] | (nvv[3] << 16));
-                    if (ADAPT || nvv[0] != sv[0] || nvv[1] != sv[1] || nvv[2] != sv[2] || nvv[3] != sv[3])
-                        *reinterpret_cast<uint2*>(st + at) = n2;
                 }
                 // Step 3b flips of the group (the single-bit variant flips after the sweep)
                 if (lane == 0 && !single) {
@@ -993,38 +1220,55 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                             if (r != S.rank) reinterpret_cast<uint4*>(peer(xw, r))[g] = nw;
                     }
                 }
-            };
-            const int full = nl >> 2, groups_l = (nl + 3) >> 2;   // only the code's last group can be partial
-            for (int gl = warp; gl < full; gl += nwarps) group(gl, std::false_type{});
-            if (full < groups_l && warp == full % nwarps) group(full, std::true_type{});
-            if constexpr (!ADAPT) {
-                // the least (E key, k) of each slot over this CTA's symbols; when split, in the
-                // buffer of this round's parity (the CTAs of the cluster read each other's)
-                unsigned long long* bcur = best + (split ? (round & 1) * kSlots : 0);
-                if (single && act) atomicMin(bcur + lane, my_best);
             }
+            if (single && act) atomicMin(bcur + lane, my_best);
         }
+        if (ADAPT || !single) break;
+        // ---- Step 3a: each decided slot flips its least-E_k symbol (the lowest k among equal
+        // values) in every copy of the decision words; every CTA of a split job sees the same
+        // minima and takes the same branches ----
         if constexpr (!ADAPT) {
-            if (!ADAPT && A.single) {
-                group_sync();
-                // each live slot flips its least-E_k symbol (the lowest k among equal values), in
-                // every copy of the decision words
-                unsigned long long* bcur = best + (split ? (round & 1) * kSlots : 0);
-                if (tid < kSlots) {
-                    unsigned long long b = bcur[tid];
-                    if constexpr (CL) {
-                        for (int r = 0; split && r < S.size; ++r) {
-                            if (r == S.rank) continue;
-                            const unsigned long long o = *peer(bcur + tid, r);
-                            b = o < b ? o : b;
+            group_sync();
+            if (warp == 0) {
+                unsigned long long b = bcur[tid];
+                if constexpr (CL) {
+                    for (int r = 0; split && r < S.size; ++r) {
+                        if (r == S.rank) continue;
+                        const unsigned long long o = *peer(bcur + tid, r);
+                        b = o < b ? o : b;
+                    }
+                }
+                const bool mine = (todo >> tid) & 1u;
+                const float least = value_of((uint32_t)(b >> 32));
+                // (with tau at infinity every symbol was evaluated: decided, even if the least is a NaN)
+                const bool found = mine && (dense || (b != ~0ull && (least <= tau[tid] || tau[tid] == INFINITY)));
+                if (found) {
+                    const int k = (int)(uint32_t)b;
+                    const bool was_neg = (atomicXor(xw + k, 1u << tid) >> tid) & 1u;
+                    if (k >= k_lo && k < k_hi) {
+                        const int at = gidx(k - k_lo, tid);
+                        if constexpr (SMOOTH) st[at] = (uint16_t)flipped_state(st[at], was_neg, round - lane_start[tid]);
+                        if constexpr (!dense) {
+                            const Job& Jf = job_of(tid);
+                            yb[at] = (uint8_t)margin_byte<PREC>(hold<PREC>(read_sample(Jf, lane_frame[tid], k), Jf),
+                                                                was_neg ? 0u : 0x80000000u, sym_deg[k - sym_base], Jf);
                         }
                     }
-                    if ((live >> tid) & 1u) atomicXor(xw + (uint32_t)b, 1u << tid);
-                    // clear the buffer of the next round (when split, the other CTAs finished
-                    // reading it before the previous round's closing barrier)
-                    best[(split ? ((round + 1) & 1) * kSlots : 0) + tid] = ~0ull;
+                    tau[tid] = least + kGuess * job_of(tid).scale;
+                    if (!split) bcur[tid] = ~0ull;
+                } else if (mine) {
+                    tau[tid] = sweep < kSweeps ? tau[tid] + kRaise * job_of(tid).scale : INFINITY;
                 }
+                // when split, the buffer of the next round (the other CTAs finished reading it
+                // before the previous round's closing barrier)
+                if (split) best[((round + 1) & 1) * kSlots + tid] = ~0ull;
+                const uint32_t left = __ballot_sync(0xFFFFFFFFu, mine && !found);
+                if (tid == 0) ctl[5] = left;
             }
+            group_sync();
+            todo = ctl[5];
+            if (todo == 0u) break;
+        }
         }
         group_sync();
         ++round;

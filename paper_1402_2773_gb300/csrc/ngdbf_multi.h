@@ -8,8 +8,8 @@
 namespace ngdbf {
 
 // The job-table kernel for a variant (NGDBF_ADAPT | NGDBF_SMOOTH | NGDBF_SINGLE), a precision,
-// the placement of the per-slot state and the count layout (4-bit lanes for symbol degrees up to
-// 7, bit slices above); usable with cudaFuncSetAttribute and the occupancy calculator.
+// the placement of the per-slot state and the count layout (4-bit counts for symbol degrees up to
+// 15, bit slices above); usable with cudaFuncSetAttribute and the occupancy calculator.
 void* multi_kernel_fn(int variant, int precision, bool st_smem, bool wide);
 
 // The same with thread-block clusters (jobs with n >= MultiArgs::split_min_n split over a cluster).

@@ -20,7 +20,7 @@ struct PlainArgs {
     int64_t n_frames;
     uint64_t frame_offset;
     const uint16_t* chk_cols;   // [dc_max][m], padded with n
-    const uint16_t* sym_chks;   // [n][dv_max], padded with m
+    const uint16_t* sym_chks;   // [n/4][dv_max][4], padded with m
     const float* y;             // [F][n]
     float w, scale, y_max;
     int32_t clamp;
@@ -137,7 +137,7 @@ __global__ void plain_update(const __grid_constant__ PlainArgs A, int t) {
             const int k = 4 * g + j;
             if (k >= A.n) break;
             int S = 0;
-            for (int d = 0; d < A.dv_max; ++d) S += sf[A.sym_chks[k * A.dv_max + d]];
+            for (int d = 0; d < A.dv_max; ++d) S += sf[A.sym_chks[(g * A.dv_max + d) * 4 + j]];
             const float yv = held_sample(A, f, k);
             const float xy = xf[k] > 0 ? yv : -yv;
             const float ws = __fmul_rn(A.w, __int2float_rn(S));

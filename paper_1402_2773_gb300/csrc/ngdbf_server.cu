@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
     __shared__ int8_t slot_e[kSlots];
     __shared__ int cur_e;
     __shared__ unsigned long long fail[2];
+    __shared__ uint32_t cut[kChain * 256];      // cutoff tables of the entries
     Job& job = jl[0];
     if (threadIdx.x == 0) fail[0] = fail[1] = ~0ull;
     __shared__ int pick;
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
         slept = 0;
         nap = 500;
         int tables = 0;
-        const ChainCtx<RingNext> ch{jl, slot_e, &cur_e, RingNext{R, fail}};
+        const ChainCtx<RingNext> ch{jl, slot_e, &cur_e, RingNext{R, fail}, cut};
         bool done = false;
         if constexpr (kState && !ST_SMEM && !WIDE) {
             const SmemLayout Ls = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT, true, WIDE,
@@ -288,7 +289,7 @@ struct Kind {
     bool fits(const ngdbf_job& q) const {
         return (q.params.variant & 3) == variant && q.params.precision == precision && q.code->n <= n &&
                q.code->m <= m && q.params.t_max <= t_max && q.code->dv_max <= dv && q.code->dc_max <= dc &&
-               ((q.code->dv_max > 7) == (dv > 7));
+               ((q.code->dv_max > kNarrowDegree) == (dv > kNarrowDegree));
     }
 };
 
@@ -437,7 +438,7 @@ struct ServePlan {
     size_t per_y = 0, per_st = 0, bytes = 0;
 };
 ngdbf_status plan_serve(ngdbf_server* S, const Kind& K, ServePlan* out) {
-    const bool state = (K.variant & 3) != 0, adapt = (K.variant & NGDBF_ADAPT) != 0, wide = K.dv > 7;
+    const bool state = (K.variant & 3) != 0, adapt = (K.variant & NGDBF_ADAPT) != 0, wide = K.dv > kNarrowDegree;
     ngdbf_status s = plan_smem(S->device, K.n, K.m, K.t_max, K.dv, K.dc, adapt, state,
                                (const void*)serve_kernel_fn(K.variant, K.precision, true, wide),
                                (const void*)serve_kernel_fn(K.variant, K.precision, false, wide), &out->sp);
@@ -455,7 +456,7 @@ ngdbf_status plan_serve(ngdbf_server* S, const Kind& K, ServePlan* out) {
 // Launches the resident kernel for the kind of the published requests (a new epoch).
 ngdbf_status launch_kernel(ngdbf_server* S) {
     const Kind& K = S->kind;
-    const bool wide = K.dv > 7;
+    const bool wide = K.dv > kNarrowDegree;
     ServePlan P;
     ngdbf_status s = plan_serve(S, K, &P);
     if (s != NGDBF_OK) return s;
@@ -502,7 +503,7 @@ Kind kind_for(ngdbf_server* S, const Request* first) {
     const ngdbf_job& f = first->job;
     Kind* K = nullptr;
     for (Kind& k : S->seen)
-        if (k.variant == (f.params.variant & 3) && k.precision == f.params.precision && (k.dv > 7) == (f.code->dv_max > 7))
+        if (k.variant == (f.params.variant & 3) && k.precision == f.params.precision && (k.dv > kNarrowDegree) == (f.code->dv_max > kNarrowDegree))
             K = &k;
     if (!K) {
         S->seen.push_back(Kind());
@@ -512,7 +513,7 @@ Kind kind_for(ngdbf_server* S, const Request* first) {
     }
     auto grow = [&](const ngdbf_job& q) {
         if ((q.params.variant & 3) != K->variant || q.params.precision != K->precision ||
-            (q.code->dv_max > 7) != (K->dv > 7 || f.code->dv_max > 7))
+            (q.code->dv_max > kNarrowDegree) != (K->dv > kNarrowDegree || f.code->dv_max > kNarrowDegree))
             return;
         K->n = std::max(K->n, q.code->n);
         K->m = std::max(K->m, q.code->m);
