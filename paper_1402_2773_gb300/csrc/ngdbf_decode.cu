@@ -369,10 +369,11 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     const SmemLayout& L = pc.L;
     const bool st_smem = pc.st_smem;
     const int placement = pc.placement;
-    const int64_t groups = (n_frames + kSlots - 1) / kSlots;
     plan->block = best_block;
     plan->blocks_per_sm = best_bps;
-    plan->grid = (int)std::min<int64_t>((int64_t)sm_count * best_bps, groups);
+    // every CTA that can be resident, as long as each gets a frame: a CTA's time per iteration
+    // grows with its live slots, so a small batch is spread over the SMs, not packed 32 to a CTA
+    plan->grid = (int)std::min<int64_t>((int64_t)sm_count * best_bps, n_frames);
     plan->smem = L.total;
     plan->st_smem = st_smem;
     plan->placement = placement;
@@ -502,9 +503,15 @@ void fill_job(const ngdbf_code* C, const ngdbf_params* P, const float* y, int64_
     fill_margins(C, P, thr, &J);
 }
 
+// Frames a CTA takes first when n_frames are decoded by n_ctas CTAs.
+int first_slots(int64_t n_frames, int64_t n_ctas) {
+    const int64_t per = (n_frames + n_ctas - 1) / std::max<int64_t>(n_ctas, 1);
+    return (int)std::min<int64_t>(std::max<int64_t>(per, 1), kSlots);
+}
+
 // Kernel arguments of one decode: scratch at `base` (work counter, then the
 // per-slot samples), per-slot state at `st_base` when it lives in global memory.
-void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& plan, const float* y,
+void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& plan, int grid, const float* y,
                int64_t n_frames, float sigma, uint64_t seed, uint64_t frame_offset, uint8_t* bits,
                int32_t* iters, uint8_t* pass, unsigned char* base, unsigned char* st_base,
                bool st_global, DecodeArgs* out) {
@@ -513,6 +520,7 @@ void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& pla
     fill_job(C, P, y, n_frames, sigma, frame_offset, bits, iters, pass,
              reinterpret_cast<unsigned long long*>(base), &A.J, A.thr);
     A.J.thr = nullptr;                 // thresholds travel inline in the launch
+    A.J.slots = first_slots(n_frames, grid);
     A.placement = plan.placement;
     A.yslots = base + 256;
     A.st_global = st_global ? reinterpret_cast<uint16_t*>(st_base) : nullptr;
@@ -606,7 +614,7 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     unsigned char* base = static_cast<unsigned char*>(ws);
 
     DecodeArgs A;
-    fill_args(C, P, plan, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
+    fill_args(C, P, plan, plan.grid, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
               base + 256 + bytes_y, bytes_st != 0, &A);
     if (tr && tr->frames > 0) {
         A.J.trace_u = tr->unsat;
@@ -990,7 +998,7 @@ extern "C" ngdbf_status ngdbf_decode_noalloc(const ngdbf_code_t* C, const float*
     const size_t bytes_y = ((size_t)grid * per_cta_y + 255) / 256 * 256;
 
     DecodeArgs A;
-    fill_args(C, P, plan, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
+    fill_args(C, P, plan, grid, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
               base + 256 + bytes_y, per_cta_st != 0, &A);
     // The work counter must start at zero; the kernel initializes everything else it reads.
     e = cudaMemsetAsync(A.J.queue, 0, sizeof(unsigned long long), stream);
@@ -1013,10 +1021,11 @@ struct ngdbf_batch {
     void* fn = nullptr;                 // job-table kernel
     int grid = 0, block = 0, smem = 0, state_in_smem = 0, tables_in_smem = 0, cluster = 1;
     MultiArgs args;
-    unsigned char* d_mem = nullptr;     // jobs | thresholds | queues | first_job | samples | state
+    unsigned char* d_mem = nullptr;     // jobs | thresholds | queues | first_job | slots | samples | state
     unsigned char* d_st = nullptr;      // per-slot state when it is not in shared memory
     unsigned long long* d_queues = nullptr;
     int32_t* d_first = nullptr;
+    int32_t* d_slots = nullptr;
     std::vector<int64_t> frames, weight;
     std::vector<int> n_of_job;
     std::vector<TableShape> shapes;
@@ -1293,9 +1302,9 @@ cudaError_t batch_enqueue(ngdbf_batch* B, cudaStream_t stream) {
     return launch_multi(B->fn, B->args, B->grid, B->block, B->smem, stream);
 }
 
-// Puts candidate `k` in use: kernel, launch shape, shared-memory plan and the first job of
-// every CTA (of every cluster: a split job keeps one cluster busy per 32 frames, a job decoded
-// CTA by CTA one cluster per 32 C frames).
+// Puts candidate `k` in use: kernel, launch shape, shared-memory plan, the first job of every CTA
+// (of every cluster: a split job can use one cluster per frame, a job decoded CTA by CTA one
+// cluster per C frames) and the frames a CTA takes first of each job.
 ngdbf_status batch_set_shape(ngdbf_batch* B, int k) {
     const TableShape& sh = B->shapes[k];
     const int C = sh.cluster;
@@ -1315,14 +1324,20 @@ ngdbf_status batch_set_shape(ngdbf_batch* B, int k) {
     std::vector<int64_t> cap(B->n_jobs);
     int64_t clusters = 0;
     for (int j = 0; j < B->n_jobs; ++j) {
-        const int64_t per = (int64_t)kSlots * (B->n_of_job[j] >= sh.split_min_n ? 1 : C);
+        const int64_t per = B->n_of_job[j] >= sh.split_min_n ? 1 : C;
         cap[j] = (B->frames[j] + per - 1) / per;
         clusters += cap[j];
     }
     const int64_t n_cl = std::max<int64_t>(1, std::min<int64_t>(sh.grid_max / C, clusters));
     B->grid = (int)(n_cl * C);
     std::vector<int32_t> first = assign_ctas_capped(B->frames, B->weight, cap, (int)n_cl);
+    std::vector<int32_t> slots(B->n_jobs, 1);
+    for (int j = 0; j < B->n_jobs; ++j) {
+        const int64_t cls = std::max<int64_t>(1, std::count(first.begin(), first.end(), j));
+        slots[j] = first_slots(B->frames[j], cls * (B->n_of_job[j] >= sh.split_min_n ? 1 : C));
+    }
     cudaError_t e = cudaMemcpy(B->d_first, first.data(), first.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(B->d_slots, slots.data(), slots.size() * 4, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "job table: first jobs");
     return NGDBF_OK;
 }
@@ -1394,7 +1409,8 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
         if (sh.state_global) bytes_st = std::max(bytes_st, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * 2);
     }
     const size_t off_jobs = 0, off_thr = align256(sizeof(Job) * n_jobs), off_q = off_thr + align256(T.thr_words * 4);
-    const size_t off_first = off_q + align256(8 * (size_t)n_jobs), off_y = off_first + align256(4 * grid_max);
+    const size_t off_first = off_q + align256(8 * (size_t)n_jobs), off_slots = off_first + align256(4 * grid_max);
+    const size_t off_y = off_slots + align256(4 * (size_t)n_jobs);
     const size_t off_st = off_y + align256(bytes_y);
     const size_t total = off_st + align256(bytes_st);
     e = cudaMalloc(&B->d_mem, total);
@@ -1405,6 +1421,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     }
     B->d_queues = reinterpret_cast<unsigned long long*>(B->d_mem + off_q);
     B->d_first = reinterpret_cast<int32_t*>(B->d_mem + off_first);
+    B->d_slots = reinterpret_cast<int32_t*>(B->d_mem + off_slots);
     B->d_st = bytes_st ? B->d_mem + off_st : nullptr;
     // job table and thresholds
     std::vector<Job> hjobs(n_jobs);
@@ -1431,6 +1448,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     A.jobs = reinterpret_cast<const Job*>(B->d_mem + off_jobs);
     A.n_jobs = n_jobs;
     A.first_job = B->d_first;
+    A.slots = B->d_slots;
     A.n_max = T.n_max; A.m_max = T.m_max; A.t_max = T.t_max; A.dv_max = T.dv_max; A.dc_max = T.dc_max;
     A.yslots = B->d_mem + off_y;
     host_gen_consts(seed, A.G);

@@ -217,6 +217,7 @@ struct MultiArgs {
     const Job* jobs;
     int32_t n_jobs;
     const int32_t* first_job;   // [grid]
+    const int32_t* slots;       // [n_jobs] Job::slots under this launch shape
     int32_t n_max, m_max, t_max, dv_max, dc_max;   // layout maxima over the jobs
     int32_t placement;          // adjacency tables copied into shared memory: kTabChk | kTabSym
     // cluster launches: jobs with n >= split_min_n are split over the `cluster` CTAs of a
@@ -365,6 +366,9 @@ __device__ __forceinline__ int select_bit(uint32_t mask, int j) {
     }
     return pos;
 }
+
+// The first `slots` slots (1..32).
+__device__ __forceinline__ uint32_t slot_mask(int slots) { return 0xFFFFFFFFu >> (kSlots - slots); }
 
 // Position of the (j+1)-th set bit of mask (j < popc(mask)).
 __device__ __forceinline__ int nth_set_bit(uint32_t mask, int j) {
@@ -690,7 +694,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if constexpr (CHAIN) {
             *ch.cur_e = 0;
             for (int f = 0; f < kSlots; ++f) ch.slot_e[f] = 0;     // every slot names a loaded entry
-            live = fill_chained(ch, A.chain_key, 0xFFFFFFFFu, 0u, 0, lane_frame, lane_start, ctl + 4);
+            live = fill_chained(ch, A.chain_key, slot_mask(A.slots), 0u, 0, lane_frame, lane_start, ctl + 4);
         } else {
             unsigned long long base = 0;
             const bool got = claim_frames(A, (unsigned)A.slots, &base);
@@ -912,7 +916,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (tid == 0 && (!split || S.rank == 0)) {
                 uint32_t fresh = 0;
                 if constexpr (CHAIN) {
-                    fresh = fill_chained(ch, A.chain_key, fin, live & ~fin, round, lane_frame, lane_start, ctl + 4);
+                    // (and the slots that a request admitted under a higher load allows)
+                    const uint32_t want = fin | (slot_mask(ch.jl[*ch.cur_e].slots) & ~live);
+                    fresh = fill_chained(ch, A.chain_key, want, live & ~fin, round, lane_frame, lane_start, ctl + 4);
                 } else {
                     unsigned long long base = 0;
                     const bool got = claim_frames(A, (unsigned)nfin, &base);

@@ -14,7 +14,10 @@ __global__ void __launch_bounds__(1024) ngdbf_multi_kernel(const __grid_constant
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_max) * kSlots : nullptr;
     int j = A.first_job[blockIdx.x];
     while (j >= 0) {
-        if (threadIdx.x == 0) job = A.jobs[j];
+        if (threadIdx.x == 0) {
+            job = A.jobs[j];
+            job.slots = A.slots[j];
+        }
         __syncthreads();
         // shared memory laid out for this job's code (the launch has room for the largest)
         int tables = 0;

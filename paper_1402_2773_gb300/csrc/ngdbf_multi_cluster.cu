@@ -22,7 +22,10 @@ __global__ void __launch_bounds__(1024) ngdbf_multi_cluster_kernel(const __grid_
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_local) * kSlots : nullptr;
     int j = A.first_job[blockIdx.x / C];
     while (j >= 0) {
-        if (threadIdx.x == 0) job = A.jobs[j];
+        if (threadIdx.x == 0) {
+            job = A.jobs[j];
+            job.slots = A.slots[j];
+        }
         __syncthreads();
         const bool sp = job.n >= A.split_min_n;
         const Split S = sp ? split_range(rank, C, job.n) : Split{0, 1, 0, job.n};
