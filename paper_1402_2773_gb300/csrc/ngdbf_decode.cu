@@ -270,7 +270,7 @@ size_t held_bytes(int precision) {
 // state stays in shared memory whenever some candidate fits with it there (it is read and
 // written for every symbol and slot); among those candidates the most resident warps per
 // SM win, then the most CTAs per SM, then more tables in shared memory (both, then the
-// N(i) table alone).  fn_of(st) gives the kernel for a state placement.  Results are cached
+// N(i) table alone, then M(k) alone).  fn_of(st) gives the kernel for a state placement.  Results are cached
 // per shape and device.
 struct PlacementChoice {
     bool st_smem = false;
@@ -302,7 +302,7 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         if (best.bps > 0) break;                       // state fits in shared memory
-        for (const int tb : {kTabChk | kTabSym, kTabChk, 0}) {
+        for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
             const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, n_local);
             if (L.total > limit) continue;
             for (const int block : {1024, 512, 256}) {
@@ -685,11 +685,11 @@ ngdbf_status ngdbf_code_create(int32_t n, int32_t m, const int32_t* row_ptr, con
         dv_max = std::max(dv_max, sdeg[k]);
     }
     if (dv_max > NGDBF_MAX_DEGREE) return fail(NGDBF_ERR_UNSUPPORTED, "symbol degree above NGDBF_MAX_DEGREE");
-    // N(i) column-major [j][i], padded with the zero-word sentinel n
-    std::vector<uint16_t> chk((size_t)dc_max * m, (uint16_t)n);
+    // N(i) in units of four (chk_index), padded with the zero-word sentinel n
+    std::vector<uint16_t> chk((size_t)m * 8 * ((dc_max + 7) / 8), (uint16_t)n);
     for (int i = 0; i < m; ++i)
-        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) chk[(size_t)(e - row_ptr[i]) * m + i] = (uint16_t)col_idx[e];
-    // M(k) by groups of four symbols [k/4][j][k%4], padded with the zero-word sentinel m, so that
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) chk[chk_index(e - row_ptr[i], i, m)] = (uint16_t)col_idx[e];
+    // M(k) by groups of four symbols [j][k/4][k%4], padded with the zero-word sentinel m, so that
     // one 8-byte load gives the j-th check of the four symbols of a group
     std::vector<uint16_t> sym((size_t)pad4(n) * dv_max, (uint16_t)m);
     std::vector<uint8_t> deg(n);
@@ -697,7 +697,7 @@ ngdbf_status ngdbf_code_create(int32_t n, int32_t m, const int32_t* row_ptr, con
     for (int i = 0; i < m; ++i)
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
             const int c = col_idx[e];
-            sym[((size_t)(c >> 2) * dv_max + fill[c]++) * 4 + (c & 3)] = (uint16_t)i;
+            sym[((size_t)fill[c]++ * (pad4(n) / 4) + (c >> 2)) * 4 + (c & 3)] = (uint16_t)i;
         }
     for (int k = 0; k < n; ++k) deg[k] = (uint8_t)sdeg[k];
 
@@ -1153,7 +1153,7 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
         void* fn = multi_kernel_fn(variant, precision, st, T.wide);
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-        for (const int tb : {kTabChk | kTabSym, kTabChk, 0}) {
+        for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
             const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, st, T.wide, tb, limit);
             if (total < 0) continue;
             for (const int block : {1024, 512, 256}) {
@@ -1209,7 +1209,7 @@ ngdbf_status table_shapes(const TablePlan& T, const ngdbf_job* jobs, int32_t n_j
         e = cudaFuncGetAttributes(&fa, T.fn);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
         const int limit = smem_optin - (int)fa.sharedSizeBytes;
-        for (const int tb : {kTabChk | kTabSym, kTabChk, 0}) {
+        for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
             if (tb == T.placement) continue;
             const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, T.st_smem, wide, tb, limit);
             if (total < 0 || total == T.smem) continue;    // no fit, or the same layouts as the plan's
@@ -1253,7 +1253,7 @@ ngdbf_status table_shapes(const TablePlan& T, const ngdbf_job* jobs, int32_t n_j
             if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFuncSetAttribute");
             bool any = false;
             int prev = -1;
-            for (const int tb : {kTabChk | kTabSym, kTabChk, 0}) {
+            for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
                 const int total = table_smem(jobs, n_jobs, C, smin, adapt, st, wide, tb, limit);
                 if (total < 0 || total == prev) continue;    // no fit, or the same layouts again
                 prev = total;

@@ -17,8 +17,8 @@
 struct ngdbf_code {
     int32_t n, m, dv_max, dc_max;
     int device;
-    uint16_t* d_chk_cols;   // [dc_max][m] N(i) column-major, padded with n
-    uint16_t* d_sym_chks;   // [n/4][dv_max][4] M(k) by groups of four symbols, padded with m
+    uint16_t* d_chk_cols;   // N(i), chk_index layout, padded with n
+    uint16_t* d_sym_chks;   // M(k), [dv_max][ceil(n / 4)][4], padded with m
     uint8_t* d_sym_deg;     // [n]
 };
 

@@ -68,6 +68,12 @@ constexpr int kSlots = 32;
 
 // Symbols rounded up to whole groups of four (the per-slot arrays are laid out by groups).
 __host__ __device__ inline int pad4(int n) { return (n + 3) & ~3; }
+// Index of the j-th symbol of N(i): units of four (one 8-byte load), two units per check side by
+// side for the two threads that share it, [j/8][i][(j/4)%2][j%4].
+__host__ __device__ inline size_t chk_index(int j, int i, int m) {
+    return (((size_t)(j >> 3) * m + i) * 2 + ((j >> 2) & 1)) * 4 + (j & 3);
+}
+__host__ __device__ inline int chk_entries(int m, int dc_max) { return m * 8 * ((dc_max + 7) >> 3); }
 // Index of (symbol k, slot f) in the group layout [k/4][slot][k%4].
 __host__ __device__ inline int gidx(int k, int f) { return (((k >> 2) * kSlots + f) << 2) | (k & 3); }
 constexpr int kTabChk = 1;              // N(i) table in shared memory
@@ -103,8 +109,8 @@ template <> struct Held<kFIXACC> { using T = int8_t; };   // the same Eq. 8 leve
 struct Job {
     // code tables (device)
     int32_t n, m, dv_max, dc_max;
-    const uint16_t* chk_cols;   // [dc_max][m]   N(i) column-major, padded with n
-    const uint16_t* sym_chks;   // [n][dv_max]   M(k) row-major, padded with m
+    const uint16_t* chk_cols;   // N(i), chk_index layout, padded with n
+    const uint16_t* sym_chks;   // M(k), [dv_max][ceil(n / 4)][4], padded with m
     const uint8_t* sym_deg;     // [n]           d_v(k)
     // batch
     const float* y;             // [n_frames][n]
@@ -294,7 +300,7 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     // don't-care but stay inside the table)
     L.off_thr = need_thr ? take((kUMask + 1) * 4, 16) : -1;
     L.off_st = st_smem ? take(pad4(n_local) * kSlots * 2, 16) : -1;
-    L.off_chk = (tables & kTabChk) ? take(dc_max * m * 2, 16) : -1;
+    L.off_chk = (tables & kTabChk) ? take(chk_entries(m, dc_max) * 2, 16) : -1;
     L.off_sym = (tables & kTabSym) ? take(pad4(n_local) * dv_max * 2 + n_local, 16) : -1;
     L.total = (o + 15) / 16 * 16;
     return L;
@@ -303,15 +309,15 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
 // Layout of one job of a job table: arrays sized for the job's own code (n_local symbols per
 // CTA: its share when split over a cluster) in the launch's count and syndrome format, with
 // as many of the adjacency tables that `tables` allows as fit in `bytes` (both, then N(i)
-// alone, then none); *tables_out receives the placement taken.  Host planning and the kernel
+// alone, M(k) alone, none); *tables_out receives the placement taken.  Host planning and the kernel
 // evaluate it alike, so the launch's shared memory is the largest job's, not the layout of
 // the table's maxima.
 __host__ __device__ inline SmemLayout job_layout(int n, int m, int t_max, int dv_max, int dc_max, bool need_thr,
                                                  bool st_smem, bool wide, int tables, int n_local, int bytes,
                                                  int* tables_out) {
-    const int opts[3] = {tables & (kTabChk | kTabSym), tables & kTabChk, 0};
+    const int opts[4] = {tables & (kTabChk | kTabSym), tables & kTabChk, tables & kTabSym, 0};
     SmemLayout L{};
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 4; ++i) {
         L = smem_layout(n, m, t_max, dv_max, dc_max, need_thr, st_smem, opts[i], n_local, wide ? 1 : 0);
         *tables_out = opts[i];
         if (L.total <= bytes) break;
@@ -488,7 +494,7 @@ __device__ __forceinline__ void trace_round(const Job& A, const SmemLayout& L, c
         const int i = base + tid;
         uint32_t s = 0u;
         if (i < m)
-            for (int j = 0; j < A.dc_max; ++j) s ^= xw[chk_cols[j * m + i]];
+            for (int j = 0; j < A.dc_max; ++j) s ^= xw[chk_cols[chk_index(j, i, m)]];
         for (uint32_t r = tmask; r; r &= r - 1u) {
             const int f = __ffs(r) - 1;
             const int c = __popc(__ballot_sync(0xFFFFFFFFu, (s >> f) & 1u));
@@ -671,18 +677,25 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     const uint8_t* sym_deg = A.sym_deg;
     if (tables & kTabChk) {
         uint16_t* c = reinterpret_cast<uint16_t*>(smem + L.off_chk);
-        for (int i = tid; i < dc_max * m; i += blockDim.x) c[i] = A.chk_cols[i];
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(A.chk_cols);
+        for (int i = tid; i < chk_entries(m, dc_max) / 2; i += blockDim.x) reinterpret_cast<uint32_t*>(c)[i] = src[i];
         chk_cols = c;
     }
-    int sym_base = 0;           // first symbol of the M(k) rows sym_chks points to
+    int sym_base = 0;           // first symbol that sym_deg (and a shared-memory M(k)) begins with
+    // M(k) in 8-byte units, one per (j, group of four symbols): the j-th checks of the four
+    int sym_groups = pad4(n) >> 2, sym_g0 = k_lo >> 2;     // units per j; unit of this CTA's first group
     if (tables & kTabSym) {
         uint16_t* s = reinterpret_cast<uint16_t*>(smem + L.off_sym);
         uint8_t* d = reinterpret_cast<uint8_t*>(s + pad4(nl) * dv_max);
-        for (int i = tid; i < pad4(nl) * dv_max; i += blockDim.x) s[i] = A.sym_chks[k_lo * dv_max + i];
+        const int gl = pad4(nl) >> 2;
+        for (int i = tid; i < gl * dv_max; i += blockDim.x)
+            reinterpret_cast<uint2*>(s)[i] = reinterpret_cast<const uint2*>(A.sym_chks)[(size_t)(i / gl) * sym_groups + sym_g0 + i % gl];
         for (int i = tid; i < nl; i += blockDim.x) d[i] = A.sym_deg[k_lo + i];
         sym_chks = s;
         sym_deg = d;
         sym_base = k_lo;
+        sym_groups = gl;
+        sym_g0 = 0;
     }
 
     // ---- the first 32 frames, then the set-up: generator table, zeroed state, sentinels,
@@ -814,24 +827,42 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             refill = false;
         }
 
-        // ---- A. syndromes (four threads XOR a quarter of a check each) and the vote ----
+        // the first checks of this thread's symbols (phase A'), fetched while the syndromes form
+        const uint2* units = reinterpret_cast<const uint2*>(sym_chks) + sym_g0;
+        const int groups_l = (nl + 3) >> 2;          // groups of four symbols (the code's last can be partial)
+        [[maybe_unused]] uint2 pre[3] = {};
+        if constexpr (!WIDE) {
+            if (tid < 2 * groups_l) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    if (d < dv_max) pre[d] = units[(size_t)d * sym_groups + (tid >> 1)];
+            }
+        }
+
+        // ---- A. syndromes (two threads XOR half of a check each) and the vote ----
         {
             uint32_t* unsat = ctl + (pass_id & 1);
             if (tid == 0) ctl[(pass_id + 1) & 1] = 0u;
             uint32_t acc = 0;
-            const int per_pass = blockDim.x >> 2, sub = tid & 3;
-            for (int base = 0; base < m; base += per_pass) {
-                const int i = base + (tid >> 2);
+            const int h = tid & 1, dc8 = (dc_max + 7) >> 3;
+            const uint2* cols = reinterpret_cast<const uint2*>(chk_cols);
+            for (int base = 0; base < m; base += blockDim.x >> 1) {
+                const int i = base + (tid >> 1);
                 uint32_t s = 0;
-                if (i < m)
-                    for (int j = sub; j < dc_max; j += 4) s ^= xw[chk_cols[j * m + i]];
+                if (i < m) {
+#pragma unroll 2
+                    for (int v = 0; v < dc8; ++v) {
+                        const uint2 c = cols[2 * (v * m + i) + h];
+                        s ^= xw[c.x & 0xFFFFu] ^ xw[c.x >> 16];
+                        s ^= xw[c.y & 0xFFFFu] ^ xw[c.y >> 16];
+                    }
+                }
                 s ^= __shfl_xor_sync(0xFFFFFFFFu, s, 1);
-                s ^= __shfl_xor_sync(0xFFFFFFFFu, s, 2);
                 if constexpr (WIDE) {
-                    if (i < m && sub == 0) sw[i] = s;
+                    if (i < m && h == 0) sw[i] = s;
                 } else {
-                    // half `sub` of the word, one slot per 2-bit lane (slots 16 sub .. 16 sub + 15)
-                    if (i < m && sub < 2) sw[2 * i + sub] = spread_pairs((s >> (16 * sub)) & 0xFFFFu);
+                    // half h of the word, one slot per 2-bit lane (slots 16 h .. 16 h + 15)
+                    if (i < m) sw[2 * i + h] = spread_pairs((s >> (16 * h)) & 0xFFFFu);
                 }
                 acc |= s;
             }
@@ -962,7 +993,6 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if (live == 0) break;
 
         // ---- A'. per symbol and slot, the count of unsatisfied checks in M(k) ----
-        const int groups_l = (nl + 3) >> 2;          // groups of four symbols (the code's last can be partial)
         // a CTA of a split job flips decisions in every copy during phase C: none before every
         // CTA has formed its syndromes (the barrier's wait is below, after the counts)
         if constexpr (CL) {
@@ -972,17 +1002,15 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             // two threads per group, each for 16 slots: the four symbols' check words added in
             // 2-bit lanes three at a time, widened to nibbles (even and odd slots), and the
             // bytes of the four symbols gathered into the words that phase C reads
-            const uint2* rows = reinterpret_cast<const uint2*>(sym_chks) + (size_t)((k_lo - sym_base) >> 2) * dv_max;
             for (int i = tid; i < 2 * groups_l; i += blockDim.x) {
                 const int gl = i >> 1, h = i & 1;
-                const uint2* row = rows + (size_t)gl * dv_max;
                 uint32_t ev[4] = {0u, 0u, 0u, 0u}, od[4] = {0u, 0u, 0u, 0u};
                 for (int e = 0; e < dv_max; e += 3) {
                     uint32_t a[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         if (e + d >= dv_max) break;
-                        const uint2 c = row[e + d];         // the d-th check of each of the four symbols
+                        const uint2 c = i == tid && e == 0 ? pre[d] : units[(size_t)(e + d) * sym_groups + gl];
                         a[0] += sw[2 * (c.x & 0xFFFFu) + h];
                         a[1] += sw[2 * (c.x >> 16) + h];
                         a[2] += sw[2 * (c.y & 0xFFFFu) + h];
@@ -1006,10 +1034,10 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         } else {
             for (int k = k_lo + tid; k < k_hi; k += blockDim.x) {
                 const int kk = k - k_lo;                      // local index of the symbol
-                const uint16_t* row = sym_chks + ((k - sym_base) >> 2) * 4 * dv_max + (k & 3);
+                const uint16_t* row = sym_chks + 4 * (size_t)(sym_g0 + (kk >> 2)) + (k & 3);
                 uint32_t b[7] = {0, 0, 0, 0, 0, 0, 0};     // count <= 127: seven slices
                 for (int e = 0; e < dv_max; ++e) {
-                    uint32_t carry = sw[row[4 * e]];
+                    uint32_t carry = sw[row[4 * (size_t)e * sym_groups]];
 #pragma unroll
                     for (int q = 0; q < 7; ++q) {
                         const uint32_t c = b[q] & carry;

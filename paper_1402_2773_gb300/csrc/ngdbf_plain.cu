@@ -19,8 +19,8 @@ struct PlainArgs {
     int32_t n, m, dv_max, dc_max, t_max, t_smooth, adapt, smooth, uniform, nb;
     int64_t n_frames;
     uint64_t frame_offset;
-    const uint16_t* chk_cols;   // [dc_max][m], padded with n
-    const uint16_t* sym_chks;   // [n/4][dv_max][4], padded with m
+    const uint16_t* chk_cols;   // chk_index layout, padded with n
+    const uint16_t* sym_chks;   // [dv_max][ceil(n / 4)][4], padded with m
     const float* y;             // [F][n]
     float w, scale, y_max;
     int32_t clamp;
@@ -73,7 +73,7 @@ __global__ void plain_syndromes(const __grid_constant__ PlainArgs A) {
         if (!A.active[f]) continue;
         const int8_t* xf = A.x + f * (A.n + 1);
         int p = 1;
-        for (int j = 0; j < A.dc_max; ++j) p *= xf[A.chk_cols[j * A.m + i]];
+        for (int j = 0; j < A.dc_max; ++j) p *= xf[A.chk_cols[chk_index(j, i, A.m)]];
         A.s[f * (A.m + 1) + i] = (int8_t)p;
         if (p < 0) atomicOr(A.unsat + f, 1u);
     }
@@ -137,7 +137,7 @@ __global__ void plain_update(const __grid_constant__ PlainArgs A, int t) {
             const int k = 4 * g + j;
             if (k >= A.n) break;
             int S = 0;
-            for (int d = 0; d < A.dv_max; ++d) S += sf[A.sym_chks[(g * A.dv_max + d) * 4 + j]];
+            for (int d = 0; d < A.dv_max; ++d) S += sf[A.sym_chks[((int64_t)d * groups + g) * 4 + j]];
             const float yv = held_sample(A, f, k);
             const float xy = xf[k] > 0 ? yv : -yv;
             const float ws = __fmul_rn(A.w, __int2float_rn(S));
