@@ -73,11 +73,9 @@ template <bool ADAPT, bool SMOOTH, bool ST_SMEM, bool WIDE, int PREC>
 __global__ void __launch_bounds__(1024) ngdbf_persistent_kernel(const __grid_constant__ DecodeArgs A) {
     using HeldT = typename Held<PREC>::T;
     const Job& J = A.J;
-    const SmemLayout L = smem_layout(J.n, J.m, J.t_max, J.dv_max, J.dc_max, ADAPT,
-                                     ST_SMEM && (ADAPT || SMOOTH), A.placement);
     HeldT* ys = static_cast<HeldT*>(A.yslots) + (size_t)blockIdx.x * pad4(J.n) * kSlots;
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(J.n) * kSlots : nullptr;
-    decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, L, A.placement, ys, st);
+    decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, with_fixed_offsets(A.L), A.placement, ys, st);
 }
 
 }  // namespace ngdbf
@@ -270,7 +268,10 @@ size_t held_bytes(int precision) {
 // state stays in shared memory whenever some candidate fits with it there (it is read and
 // written for every symbol and slot); among those candidates the most resident warps per
 // SM win, then the most CTAs per SM, then more tables in shared memory (both, then the
-// N(i) table alone, then M(k) alone).  fn_of(st) gives the kernel for a state placement.  Results are cached
+// N(i) table alone, then M(k) alone).  With `many` frames (enough for two CTAs of 32 slots per
+// SM) the state, which only flips touch, goes to global memory where that puts two CTAs on an
+// SM: one computes while the other waits at a barrier or for the exact form's samples ((6,32)
+// N=2048: 200000 frames at 3.5 dB 215 -> 196 ms, 60000 FP16 at 4 dB 25.4 -> 22.9 ms).  fn_of(st) gives the kernel for a state placement.  Results are cached
 // per shape and device.
 struct PlacementChoice {
     bool st_smem = false;
@@ -280,11 +281,11 @@ struct PlacementChoice {
 
 template <class FnOf>
 ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int dc_max, bool adapt, bool state,
-                              int limit, FnOf fn_of, PlacementChoice* out, int n_local = -1) {
+                              int limit, FnOf fn_of, PlacementChoice* out, int n_local = -1, bool many = false) {
     using Key = std::vector<int64_t>;
     static std::mutex mu;
     static std::map<Key, PlacementChoice> cache;
-    const Key key = {dev, n, m, t_max, dv_max, dc_max, adapt, state, limit, n_local,
+    const Key key = {dev, n, m, t_max, dv_max, dc_max, adapt, state, limit, n_local, many,
                      (int64_t)(intptr_t)fn_of(true), (int64_t)(intptr_t)fn_of(false)};
     {
         std::lock_guard<std::mutex> g(mu);
@@ -301,7 +302,10 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
         const void* fn = fn_of(st);
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-        if (best.bps > 0) break;                       // state fits in shared memory
+        // state fits in shared memory: kept there, unless the batch fills more CTAs and without it two
+        // CTAs of 512 threads or more share an SM
+        if (best.bps > 0 && !(many && best.bps == 1)) break;
+        const bool second = best.bps > 0;
         for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
             const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, n_local);
             if (L.total > limit) continue;
@@ -310,6 +314,7 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, block, L.total);
                 if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
                 const int warps = bps * block / 32;
+                if (second && !(bps > 1 && block >= 512)) continue;
                 if (bps > 0 && (warps > best_warps || (warps == best_warps && bps > best.bps))) {
                     best_warps = warps;
                     best.st_smem = st;
@@ -350,7 +355,7 @@ ngdbf_status plan_smem(int dev, int n, int m, int t_max, int dv_max, int dc_max,
 }
 
 ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_frames, int dev,
-                         LaunchPlan* plan, KernelFn* fn_out, int* sm_count_out) {
+                         LaunchPlan* plan, KernelFn* fn_out, int* sm_count_out, bool scarce_scratch = false) {
     int sm_count = 0, smem_optin = 0, smem_per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -360,9 +365,10 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     const bool adapt = (P->variant & NGDBF_ADAPT) != 0;
     const bool wide = C->dv_max > kNarrowDegree;
     PlacementChoice pc;
+    const bool many = !wide && !scarce_scratch && n_frames >= 2ll * sm_count * kSlots;
     ngdbf_status s = choose_placement(dev, C->n, C->m, P->t_max, C->dv_max, C->dc_max, adapt, state, smem_optin,
                                       [&](bool st) { return (const void*)pick_kernel(P->variant, P->precision, st, wide); },
-                                      &pc);
+                                      &pc, -1, many);
     if (s != NGDBF_OK) return s;
     KernelFn fn = pick_kernel(P->variant, P->precision, pc.st_smem, wide);
     const int best_block = pc.block, best_bps = pc.bps;
@@ -522,6 +528,8 @@ void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& pla
     A.J.thr = nullptr;                 // thresholds travel inline in the launch
     A.J.slots = first_slots(n_frames, grid);
     A.placement = plan.placement;
+    A.L = smem_layout(C->n, C->m, P->t_max, C->dv_max, C->dc_max, (P->variant & NGDBF_ADAPT) != 0,
+                      plan.st_smem && (P->variant & 3) != 0, plan.placement);
     A.yslots = base + 256;
     A.st_global = st_global ? reinterpret_cast<uint16_t*>(st_base) : nullptr;
     host_gen_consts(seed, A.G);
@@ -603,7 +611,7 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     const size_t slot_elems = (size_t)plan.grid * pad4(C->n) * kSlots;
     const size_t bytes_y = (slot_elems * held_bytes(P->precision) + 255) / 256 * 256;
     const size_t bytes_st = (state && !plan.st_smem) ? (slot_elems * 2 + 255) / 256 * 256 : 0;
-    const size_t total = 256 + bytes_y + bytes_st;
+    const size_t total = 256 + bytes_y + bytes_st + kMarginSlack;
     void* ws = nullptr;
     e = cudaMallocFromPoolAsync(&ws, total, pool, stream);
     if (e != cudaSuccess) {
@@ -981,14 +989,14 @@ extern "C" ngdbf_status ngdbf_decode_noalloc(const ngdbf_code_t* C, const float*
     LaunchPlan plan;
     KernelFn fn;
     int sm_count = 0;
-    s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count);
+    s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count, true);
     if (s != NGDBF_OK) return s;
 
     // Fit the launch into the static array: fewer CTAs when a full grid does not fit.
     const bool state = (P->variant & 3) != 0;
     const size_t per_cta_y = (size_t)pad4(C->n) * kSlots * held_bytes(P->precision);
     const size_t per_cta_st = (state && !plan.st_smem) ? (size_t)pad4(C->n) * kSlots * 2 : 0;
-    const size_t avail = (size_t)NGDBF_NOALLOC_SCRATCH_BYTES - 256 - 256;   // counter + alignment
+    const size_t avail = (size_t)NGDBF_NOALLOC_SCRATCH_BYTES - 256 - 256 - kMarginSlack;   // counter, alignment
     const size_t max_grid = avail / (per_cta_y + per_cta_st);
     if (max_grid < 1)
         return fail(NGDBF_ERR_UNSUPPORTED, "code needs more per-CTA scratch (" +
@@ -1412,7 +1420,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     const size_t off_first = off_q + align256(8 * (size_t)n_jobs), off_slots = off_first + align256(4 * grid_max);
     const size_t off_y = off_slots + align256(4 * (size_t)n_jobs);
     const size_t off_st = off_y + align256(bytes_y);
-    const size_t total = off_st + align256(bytes_st);
+    const size_t total = off_st + align256(bytes_st) + kMarginSlack;
     e = cudaMalloc(&B->d_mem, total);
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -20,6 +20,10 @@
 //      it are queued and only for those E_k = x_k y_k + w S_k + q_k is formed and
 //      compared with theta lambda^{u_k} (Step 3a: with the slot's least so far).  Symbol
 //      degrees above 15 form E_k for every symbol, with lane = slot.
+// When an iteration flipped few decisions (at most kFlips, a code not split over a cluster),
+// A and A' are replaced by
+//   D. per flip, its d_v checks toggled for the slot, the slot's number of unsatisfied checks
+//      and the counts of the checks' symbols moved by one.
 // Slots therefore iterate independently (each frame has its own t), a
 // converged frame frees its slot at once, and the CTA only stops when the
 // queue is empty and its last slot finished.
@@ -88,7 +92,11 @@ constexpr int kNarrowDegree = 15;     // largest symbol degree of the 4-bit coun
 // evaluated), pf_K d_v is at most kMarginCounts and pf_K d_v + D(t) at most kMargin0, so that
 // no byte of a group borrows from or carries into another.
 constexpr int kMargin0 = 96, kMarginCounts = 80;
-constexpr int kQueue = 32;            // outputs queued per warp for the exact form
+// Most flips of one iteration of a CTA by which the syndromes and counts are moved (D).
+constexpr int kFlips = 256;
+// Bytes readable past a CTA's margin bytes (the last step of phase C reads whole warps of groups).
+constexpr int kMarginSlack = 32 * 32 * 4;
+constexpr int kQueue = 64;            // groups queued per warp for the exact form
 // Single-bit: the least E_k is guessed kGuess noise scales above the last, the first kFirst above
 // the lowest tau followed, raised by kRaise at a time and to infinity after kSweeps sweeps.
 constexpr float kGuess = 1.5f, kFirst = 2.0f, kRaise = 2.0f;
@@ -205,12 +213,19 @@ __device__ __forceinline__ bool claim_frames(const Job& A, unsigned k, unsigned 
     return false;
 }
 
+// Offsets in bytes of the shared-memory arrays (smem_layout).
+struct SmemLayout {
+    int32_t off_frame, off_start, off_ctl, off_unsat, off_flips, off_best, off_tau, off_trace, off_icdf, off_cut, off_queue, off_xw, off_sw, off_cnt,
+        off_thr, off_st, off_chk, off_sym, total;
+};
+
 // Launch of one job: the job and its thresholds travel as kernel parameters.
 struct DecodeArgs {
     Job J;
     int32_t placement;          // adjacency tables copied into shared memory: kTabChk | kTabSym
     void* yslots;               // [grid][pad4(n)/4][32][4] held samples (4, 2 or 1 bytes each)
     uint16_t* st_global;        // [grid][pad4(n)/4][32][4] when the state is not in shared memory
+    SmemLayout L;
     GenConsts G;
     uint32_t thr[kMaxT + 1];
 };
@@ -254,13 +269,11 @@ __host__ __device__ inline Split split_range(int rank, int size, int n) {
 // Largest number of symbols a CTA holds when a code of n symbols is split over `size` CTAs.
 __host__ __device__ inline int split_local_max(int n, int size) { return 32 * (((n + 31) / 32 + size - 1) / size); }
 
-struct SmemLayout {
-    int32_t off_frame, off_start, off_ctl, off_best, off_tau, off_trace, off_icdf, off_cut, off_queue, off_xw, off_sw, off_cnt,
-        off_thr, off_st, off_chk, off_sym, total;
-};
 
-// Offsets in bytes of the shared-memory arrays.  ctl holds: [0..1] unsatisfied
-// masks (double-buffered by pass parity), [2] live mask, [3] new-slot mask.
+// Offsets in bytes of the shared-memory arrays (-1: not placed).  ctl holds: [0..1] unsatisfied
+// masks (double-buffered by pass parity; wide and split jobs), [2] live mask, [3] new-slot
+// mask, [4] chain entries loaded, [5] single-bit slots left, [6..7] flips of this iteration
+// (double-buffered by round parity).
 // When d_v <= 15 (narrow), sw holds per check two words with one 2-bit lane per slot (lane
 // f & 15 of word f >> 4: 1 when check i is unsatisfied for slot f), and cnt holds per group of
 // four symbols sixteen words of their counts of unsatisfied checks: byte k % 4 of word
@@ -287,13 +300,17 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     L.off_frame = take(kSlots * 8, 16);
     L.off_start = take(kSlots * 4, 16);
     L.off_ctl = take(8 * 4, 16);
+    L.off_unsat = take(kSlots * 4, 16);    // number of unsatisfied checks of each slot
+    L.off_flips = take(kFlips * 4, 16);    // flips of this iteration: local symbol | slot << 16
     L.off_best = take(2 * kSlots * 8, 16); // single-bit variant: least (E key, k) per slot, two rounds
     L.off_tau = take(kSlots * 4, 16);      // single-bit variant: guess of each slot's least E_k
     L.off_trace = take(kSlots * 12, 16);   // objective trace: per slot C (int64), then U (int32)
     L.off_icdf = take(256 * 16, 16);       // inverse normal CDF coefficients
     L.off_cut = take(256 * 4, 16);         // cutoff of each margin byte
-    L.off_queue = take(32 * kQueue * 8, 16);   // per warp: outputs for the exact form
     L.off_cnt = take(pad4(n_local) * cnt_bytes, 16);
+    // per warp: groups for the exact form (phase C's last steps may read up to 31 groups of counts
+    // past the code's: they lie inside this array)
+    L.off_queue = take(32 * kQueue * 4, 16);
     L.off_xw = take(pad4(n + 1) * 4, 16);
     L.off_sw = take((m + 1) * (wd ? 4 : 8), 16);
     // all 512 values of the 9-bit u field: an idle slot's counter may pass T (its lookups are
@@ -303,6 +320,24 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     L.off_chk = (tables & kTabChk) ? take(chk_entries(m, dc_max) * 2, 16) : -1;
     L.off_sym = (tables & kTabSym) ? take(pad4(n_local) * dv_max * 2 + n_local, 16) : -1;
     L.total = (o + 15) / 16 * 16;
+    return L;
+}
+
+// Layout L with the offsets that do not depend on the code (all up to the counts) as compile-time
+// constants.
+__device__ __forceinline__ SmemLayout with_fixed_offsets(SmemLayout L) {
+    const SmemLayout F = smem_layout(4, 1, 0, 1, 1, false, false, 0);
+    L.off_frame = F.off_frame;
+    L.off_start = F.off_start;
+    L.off_ctl = F.off_ctl;
+    L.off_unsat = F.off_unsat;
+    L.off_flips = F.off_flips;
+    L.off_best = F.off_best;
+    L.off_tau = F.off_tau;
+    L.off_trace = F.off_trace;
+    L.off_icdf = F.off_icdf;
+    L.off_cut = F.off_cut;
+    L.off_cnt = F.off_cnt;
     return L;
 }
 
@@ -375,6 +410,18 @@ __device__ __forceinline__ int select_bit(uint32_t mask, int j) {
 
 // The first `slots` slots (1..32).
 __device__ __forceinline__ uint32_t slot_mask(int slots) { return 0xFFFFFFFFu >> (kSlots - slots); }
+
+// Lane f receives the number of lanes whose word has bit f set (a 32 x 32 bit transpose).
+__device__ __forceinline__ int column_count(uint32_t s, int lane) {
+    uint32_t mask = 0x0000FFFFu;
+#pragma unroll
+    for (int j = 16; j; j >>= 1) {
+        const uint32_t t = __shfl_xor_sync(0xFFFFFFFFu, s, j);
+        s = (lane & j) ? (s & ~mask) | ((t & ~mask) >> j) : (s & mask) | ((t & mask) << j);
+        mask ^= mask << (j >> 1);
+    }
+    return __popc(s);
+}
 
 // Position of the (j+1)-th set bit of mask (j < popc(mask)).
 __device__ __forceinline__ int nth_set_bit(uint32_t mask, int j) {
@@ -653,6 +700,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     long long* lane_frame = reinterpret_cast<long long*>(smem + L.off_frame);
     int32_t* lane_start = reinterpret_cast<int32_t*>(smem + L.off_start);
     uint32_t* ctl = reinterpret_cast<uint32_t*>(smem + L.off_ctl);
+    int32_t* unsat_n = reinterpret_cast<int32_t*>(smem + L.off_unsat);
+    uint32_t* flips = reinterpret_cast<uint32_t*>(smem + L.off_flips);
     uint4* cnt = reinterpret_cast<uint4*>(smem + L.off_cnt);
     uint32_t* xw = reinterpret_cast<uint32_t*>(smem + L.off_xw);
     uint32_t* sw = reinterpret_cast<uint32_t*>(smem + L.off_sw);
@@ -663,13 +712,20 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     const bool single = !ADAPT && A.single;
     // wide: every symbol evaluated, with its held sample in `ys`; else margin bytes there
     constexpr bool dense = WIDE;
+    // syndromes and counts kept between iterations and moved by the flips when these are few
+    const bool keep = !WIDE && !split;
+    // (D: lanes per check of a flip, and the flips up to which it is used: its shared atomics, a
+    // warp instruction per 32 lanes, against the n d_v edges of A and A')
+    const int sg_log = dc_max > 16 ? 5 : (dc_max > 1 ? 32 - __clz(dc_max - 1) : 0);
+    const int few = min(kFlips, n * dv_max / (32 * (((dv_max << sg_log) + 31) >> 5)));
     uint8_t* yb = reinterpret_cast<uint8_t*>(ys);
     uint32_t* thr = ADAPT ? reinterpret_cast<uint32_t*>(smem + L.off_thr) : nullptr;
     uint16_t* st = nullptr;
     if constexpr (kState) {
         st = ST_SMEM ? reinterpret_cast<uint16_t*>(smem + L.off_st) : st_cta;
     }
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, nwarps = blockDim.x >> 5, nw_log = 31 - __clz(nwarps);
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);      // uniform, and known to be
     // adjacency tables: only phases A and A' read them, so a generic pointer to
     // shared or global memory serves both placements
     const uint16_t* chk_cols = A.chk_cols;
@@ -747,8 +803,6 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     // threshold of the non-adaptive variants; chained jobs read it once here, since the first
     // job's memory is returned when that job completes
     const uint32_t th0_once = CHAIN ? __ldcg(thr_src) : 0u;
-    if constexpr (kState)
-        for (int e = tid; e < pad4(nl) * kSlots; e += blockDim.x) st[e] = 0;
     if (tid < 2 * kSlots) best[tid] = ~0ull;
     if (split) {
         group_sync();        // every copy cleared before rank 0 writes the slot table
@@ -776,6 +830,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     int round = 0;   // flip phases executed by this CTA; slot f is at t = round - lane_start[f]
     int pass_id = 0;
     bool refill = true;
+    bool anew = true;   // syndromes and counts formed from the decisions (else kept, D)
     for (;;) {
         if (refill) {
             // ---- load new frames: saturated samples into the slot columns, x(0) = sign(y) ----
@@ -825,25 +880,30 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             group_sync();
             if (CHAIN && tid == 0) ctl[4] = 0u;
             refill = false;
+            anew = true;
         }
 
-        // the first checks of this thread's symbols (phase A'), fetched while the syndromes form
         const uint2* units = reinterpret_cast<const uint2*>(sym_chks) + sym_g0;
         const int groups_l = (nl + 3) >> 2;          // groups of four symbols (the code's last can be partial)
         [[maybe_unused]] uint2 pre[3] = {};
-        if constexpr (!WIDE) {
-            if (tid < 2 * groups_l) {
+        if (anew) {
+            // the first checks of this thread's symbols (phase A'), fetched while the syndromes form
+            if constexpr (!WIDE) {
+                if (tid < 2 * groups_l) {
 #pragma unroll
-                for (int d = 0; d < 3; ++d)
-                    if (d < dv_max) pre[d] = units[(size_t)d * sym_groups + (tid >> 1)];
+                    for (int d = 0; d < 3; ++d)
+                        if (d < dv_max) pre[d] = units[(size_t)d * sym_groups + (tid >> 1)];
+                }
             }
-        }
-
-        // ---- A. syndromes (two threads XOR half of a check each) and the vote ----
-        {
+            // ---- A. syndromes (two threads XOR half of a check each) and the vote ----
             uint32_t* unsat = ctl + (pass_id & 1);
             if (tid == 0) ctl[(pass_id + 1) & 1] = 0u;
+            if (keep) {
+                if (tid < kSlots) unsat_n[tid] = 0;
+                __syncthreads();
+            }
             uint32_t acc = 0;
+            int open = 0;                // unsatisfied checks of slot `lane` seen by this warp
             const int h = tid & 1, dc8 = (dc_max + 7) >> 3;
             const uint2* cols = reinterpret_cast<const uint2*>(chk_cols);
             for (int base = 0; base < m; base += blockDim.x >> 1) {
@@ -864,14 +924,19 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                     // half h of the word, one slot per 2-bit lane (slots 16 h .. 16 h + 15)
                     if (i < m) sw[2 * i + h] = spread_pairs((s >> (16 * h)) & 0xFFFFu);
                 }
-                acc |= s;
+                if (keep) open += column_count(h ? 0u : s, lane);
+                else acc |= s;
             }
-            acc = __reduce_or_sync(0xFFFFFFFFu, acc);
-            if (lane == 0 && acc) atomicOr(unsat, acc);
+            if (keep) {
+                if (open) atomicAdd(unsat_n + lane, open);
+            } else {
+                acc = __reduce_or_sync(0xFFFFFFFFu, acc);
+                if (lane == 0 && acc) atomicOr(unsat, acc);
+            }
             __syncthreads();
         }
-        const uint32_t unsat = ctl[pass_id & 1];
-        ++pass_id;
+        const uint32_t unsat = keep ? __ballot_sync(0xFFFFFFFFu, unsat_n[lane] != 0) : ctl[pass_id & 1];
+        if (anew) ++pass_id;
         uint32_t live = ctl[2];
         if (A.trace_u != nullptr)
             trace_round<PREC>(A, L, chk_cols, live, round);
@@ -993,6 +1058,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if (live == 0) break;
 
         // ---- A'. per symbol and slot, the count of unsatisfied checks in M(k) ----
+        uint32_t* n_flips = ctl + 6 + (round & 1);
+        if (tid == 0) ctl[6 + ((round + 1) & 1)] = 0u;
+        if (anew) {
         // a CTA of a split job flips decisions in every copy during phase C: none before every
         // CTA has formed its syndromes (the barrier's wait is below, after the counts)
         if constexpr (CL) {
@@ -1053,6 +1121,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (split) cooperative_groups::this_cluster().barrier_wait();
         }
         __syncthreads();
+        }
 
         // threshold of the non-adaptive variants
         const uint32_t th0 = CHAIN ? th0_once : (A.gen ? __ldcg(thr_src) : thr_src[0]);
@@ -1089,9 +1158,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         // ---- C. Step 2 and Step 3b for every symbol of every live slot ----
         for (int sweep = 1;; ++sweep) {
         if constexpr (!dense) {
-            // lanes over (group, slot): `per` groups at a time when few slots are live
+            // lanes over (group, slot): several groups at a time when few slots are live
             const int n_live = __popc(todo);
-            const int lg = n_live > 1 ? 32 - __clz(n_live - 1) : 0, per = 32 >> lg;
+            const int lg = n_live > 1 ? 32 - __clz(n_live - 1) : 0;
             const int li = lane & ((1 << lg) - 1);
             const bool act = li < n_live;
             const int slot = n_live == 32 ? lane : select_bit(todo, act ? li : 0);
@@ -1109,85 +1178,147 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             }
             if constexpr (CHAIN) ebase = (uint32_t)ch.slot_e[slot];
             const uint32_t csh = (uint32_t)cnt_shift(slot);
-            const uint32_t* yrow = reinterpret_cast<const uint32_t*>(yb) + slot;
-            const uint32_t* crow = cntw + cnt_word(slot);
-            uint2* queue = reinterpret_cast<uint2*>(smem + L.off_queue) + warp * kQueue;
+            // queue: local group | slot << 16 | outputs at or below their cutoffs << 24
+            uint32_t* queue = reinterpret_cast<uint32_t*>(smem + L.off_queue) + warp * kQueue;
             int queued = 0;
 
-            // the exact form for the queued outputs, one per lane
-            auto evaluate = [&](int count) {
-                __syncwarp();
-                if (lane < count) {
-                    const uint2 q = queue[lane];
-                    const int kl = (int)(q.y & 0xFFFFu), f = (int)(q.y >> 16), k = k_lo + kl;
-                    if (k < k_hi) {
-                        const Job& Jf = job_of(f);
-                        const HeldT h = hold<PREC>(read_sample(Jf, lane_frame[f], k), Jf);
-                        const int tf = round - lane_start[f];
-                        const int deg = sym_deg[k - sym_base];
-                        const uint32_t c = (cntw[(kl >> 2) * 16 + cnt_word(f)] >> (8 * (kl & 3) + cnt_shift(f))) & 0xFu;
-                        uint32_t* xk = xw + k;
-                        const uint32_t xsign = ((*(volatile uint32_t*)xk >> f) & 1u) << 31;
-                        const float z = uniform ? uniform_dev(q.x) : gauss_icdf(q.x, icdf);
-                        const auto E = metric<PREC>(h, xsign, deg - 2 * (int)c, __fmul_rn(Jf.scale, z), A);
-                        if (single) {
-                            // Step 3a: the slot's least E_k (the lowest k among equal values)
-                            const unsigned long long cand = ((unsigned long long)key_of(E) << 32) | (uint32_t)k;
-                            if (cand < *(volatile unsigned long long*)(bcur + f)) atomicMin(bcur + f, cand);
-                        } else {
-                            const int at = gidx(kl, f);
-                            [[maybe_unused]] uint32_t s0 = 0u;
-                            if constexpr (kState) s0 = st[at];
-                            if (below<PREC>(E, ADAPT ? thr[(tf - (int)(s0 & kUMask)) & kUMask] : th0)) {
-                                atomicXor(xk, 1u << f);
-                                if constexpr (CL) {
-                                    for (int r = 0; split && r < S.size; ++r)
-                                        if (r != S.rank) atomicXor(peer(xw, r) + k, 1u << f);
-                                }
-                                if constexpr (kState) st[at] = (uint16_t)flipped_state(s0, xsign != 0u, tf);
-                                yb[at] = (uint8_t)margin_byte<PREC>(h, xsign ^ 0x80000000u, deg, Jf);
+            // the exact form for one output of one symbol per lane that is `on`: E_k, its flip (or, in the
+            // single-bit variant, its claim to be the slot's least)
+            auto settle = [&](bool on, int kl, int f, uint32_t out) {
+                bool flip = false;
+                const int k = k_lo + kl;
+                if (on && k < k_hi) {
+                    const Job& Jf = job_of(f);
+                    const HeldT h = hold<PREC>(read_sample(Jf, lane_frame[f], k), Jf);
+                    const int tf = round - lane_start[f];
+                    const int deg = sym_deg[k - sym_base];
+                    const uint32_t c = (cntw[(kl >> 2) * 16 + cnt_word(f)] >> (8 * (kl & 3) + cnt_shift(f))) & 0xFu;
+                    uint32_t* xk = xw + k;
+                    const uint32_t xsign = ((*(volatile uint32_t*)xk >> f) & 1u) << 31;
+                    const float z = uniform ? uniform_dev(out) : gauss_icdf(out, icdf);
+                    const auto E = metric<PREC>(h, xsign, deg - 2 * (int)c, __fmul_rn(Jf.scale, z), A);
+                    if (single) {
+                        // Step 3a: the slot's least E_k (the lowest k among equal values)
+                        const unsigned long long cand = ((unsigned long long)key_of(E) << 32) | (uint32_t)k;
+                        if (cand < *(volatile unsigned long long*)(bcur + f)) atomicMin(bcur + f, cand);
+                    } else {
+                        const int at = gidx(kl, f);
+                        [[maybe_unused]] uint32_t s0 = 0u;
+                        if constexpr (kState) s0 = st[at];
+                        flip = below<PREC>(E, ADAPT ? thr[(tf - (int)(s0 & kUMask)) & kUMask] : th0);
+                        if (flip) {
+                            atomicXor(xk, 1u << f);
+                            if constexpr (CL) {
+                                for (int r = 0; split && r < S.size; ++r)
+                                    if (r != S.rank) atomicXor(peer(xw, r) + k, 1u << f);
                             }
+                            if constexpr (kState) st[at] = (uint16_t)flipped_state(s0, xsign != 0u, tf);
+                            yb[at] = (uint8_t)margin_byte<PREC>(h, xsign ^ 0x80000000u, deg, Jf);
                         }
                     }
                 }
+                // recorded while they are few enough to be used (D)
+                const uint32_t fl = __ballot_sync(0xFFFFFFFFu, flip);
+                if (fl && keep && *(volatile uint32_t*)n_flips <= (uint32_t)few) {
+                    int at = 0;
+                    if (lane == 0) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
+                    at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(fl & ((1u << lane) - 1u));
+                    if (flip && at < kFlips) flips[at] = (uint32_t)kl | ((uint32_t)f << 16);
+                }
+            };
+            // the exact form for the first marked output of the last `count` queued groups, one group
+            // per lane (its outputs drawn again: four bytes queued instead of twenty, and nothing of
+            // the draw kept in the sweep); groups with further marks go back into the queue
+            auto evaluate = [&](int count) {
+                __syncwarp();
+                queued -= count;
+                const uint32_t q = lane < count ? queue[queued + lane] : 0u;
+                const int f = q ? (int)((q >> 16) & 31u) : slot, j = (__ffs(q >> 24) - 1) & 3, g = (int)(q & 0xFFFFu);
+                uint32_t r[4];
+                PhiloxLane(job_of(f).frame_offset + (uint64_t)lane_frame[f], (uint32_t)(round - lane_start[f]), G)
+                    .group((uint32_t)(g_lo + g), G, r);
+                settle(q != 0u, 4 * g + j, f, j & 2 ? (j & 1 ? r[3] : r[2]) : (j & 1 ? r[1] : r[0]));
+                uint32_t rest = q & ~(1u << (24 + j));
+                if ((rest >> 24) == 0u) rest = 0u;
+                const uint32_t back = __ballot_sync(0xFFFFFFFFu, rest != 0u);
+                if (rest) queue[queued + __popc(back & ((1u << lane) - 1u))] = rest;
+                queued += __popc(back);
                 __syncwarp();
             };
 
-            for (int g0 = warp * per; g0 < groups_l; g0 += nwarps * per) {
-                const int gl = g0 + (lane >> lg);
-                const bool ok = act && gl < groups_l;
-                const int gs = ok ? gl : 0;
-                // the loads before the generator's arithmetic, so that their latency overlaps it
-                const uint32_t y4 = yrow[gs * kSlots], c4 = crow[gs * 16];
-                uint32_t r[4];
-                ph.group((uint32_t)(g_lo + gs), G, r);
-                const uint32_t m4 = y4 + D - K * ((c4 >> csh) & 0x0F0F0F0Fu);
-                bool low[4];
+            // Steps of one or more groups, a contiguous range of them per warp (the lanes past the code's
+            // last group or without a slot compute on what they read and are masked where outputs are
+            // queued).  With every lane on a slot of its own (ALL) a step is one group, the strides are
+            // constants, the first generator rounds' products of the group uniform, and two steps go
+            // together for their independent chains; with fewer slots there are few steps per warp.
+            auto run = [&](auto all_tag) {
+                constexpr bool ALL = decltype(all_tag)::value;
+                constexpr int U = ALL ? 2 : 1;
+                const int lgs = ALL ? 5 : lg, stride = 1 << (5 - lgs);
+                const int steps = (groups_l + stride - 1) >> (5 - lgs);
+                const int each = ((steps + U * nwarps - 1) >> (nw_log + U - 1)) * U;
+                const int s_end = min((warp + 1) * each, steps);
+                int gl = ((warp * each) << (5 - lgs)) + (ALL ? 0 : lane >> lgs);
+                const uint32_t* yp = reinterpret_cast<const uint32_t*>(yb) + (size_t)gl * kSlots + slot;
+                const uint32_t* cp = cntw + gl * 16 + cnt_word(slot);
+                for (int step = warp * each; step < s_end; step += U) {
+                    // the loads before the generator's arithmetic, so that their latency overlaps it
+                    uint32_t y4[U], c4[U], r[U][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    uint32_t i = __byte_perm(m4, ebase, 0x5540 + j);
-                    if (single) i = (i & ~0xFFu) | (uint32_t)max((int)(i & 0xFFu) + shift, 0);
-                    low[j] = r[j] <= cut[i];
-                }
-                if (__any_sync(0xFFFFFFFFu, ok && (low[0] || low[1] || low[2] || low[3]))) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool mine = ok && low[j];
-                        const uint32_t b = __ballot_sync(0xFFFFFFFFu, mine);
-                        if (b == 0u) continue;
-                        const int more = __popc(b);
-                        if (queued + more > kQueue) {
-                            evaluate(queued);
-                            queued = 0;
-                        }
-                        if (mine)
-                            queue[queued + __popc(b & ((1u << lane) - 1u))] =
-                                make_uint2(r[j], (uint32_t)(4 * gl + j) | ((uint32_t)slot << 16));
-                        queued += more;
+                    for (int u = 0; u < U; ++u) {
+                        y4[u] = yp[u * stride * kSlots];
+                        c4[u] = cp[u * stride * 16];
                     }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) ph.group((uint32_t)(g_lo + gl + u * stride), G, r[u]);
+                    bool low[U][4], any = false;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const uint32_t m4 = y4[u] + D - K * ((c4[u] >> csh) & 0x0F0F0F0Fu);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            uint32_t i = __byte_perm(m4, ebase, 0x5540 + j);
+                            if (single) i = (i & ~0xFFu) | (uint32_t)max((int)(i & 0xFFu) + shift, 0);
+                            low[u][j] = r[u][j] <= cut[i];
+                            any = any || low[u][j];
+                        }
+                    }
+                    if (__any_sync(0xFFFFFFFFu, any)) {
+                        uint32_t mark[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            mark[u] = (low[u][0] ? 1u : 0u) | (low[u][1] ? 2u : 0u) | (low[u][2] ? 4u : 0u) | (low[u][3] ? 8u : 0u);
+                            if (!(act && step + u < s_end && gl + u * stride < groups_l)) mark[u] = 0u;
+                        }
+                        if (ALL || each > 2) {
+#pragma unroll 1
+                            for (int u = 0; u < U; ++u) {
+                                const uint32_t mk = u ? mark[U - 1] : mark[0];
+                                const uint32_t b = __ballot_sync(0xFFFFFFFFu, mk != 0u);
+                                if (mk)
+                                    queue[queued + __popc(b & ((1u << lane) - 1u))] =
+                                        (uint32_t)(gl + u * stride) | ((uint32_t)slot << 16) | (mk << 24);
+                                queued += __popc(b);
+                                while (queued >= 32) evaluate(32);
+                            }
+                        } else {
+                            // few steps per warp: its own outputs at once, for the shorter way to the barrier
+                            uint32_t mk = mark[0];
+                            while (__any_sync(0xFFFFFFFFu, mk != 0u)) {
+                                const int j = (__ffs(mk) - 1) & 3;
+                                settle(mk != 0u, 4 * gl + j, slot, j & 2 ? (j & 1 ? r[0][3] : r[0][2]) : (j & 1 ? r[0][1] : r[0][0]));
+                                mk &= mk - 1u;
+                            }
+                        }
+                    }
+                    gl += U * stride;
+                    yp += U * stride * kSlots;
+                    cp += U * stride * 16;
                 }
-            }
-            if (queued) evaluate(queued);
+            };
+            if (lg == 5) run(std::true_type{});
+            else run(std::false_type{});
+            while (queued) evaluate(queued < 32 ? queued : 32);
         } else {
             // every symbol of every slot, lane = slot (an idle slot's decisions and counters are
             // don't-care: cleared when it takes a frame, never part of an output)
@@ -1288,6 +1419,10 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                                                                 was_neg ? 0u : 0x80000000u, sym_deg[k - sym_base], Jf);
                         }
                     }
+                    if (keep) {
+                        const int at = (int)atomicAdd(n_flips, 1u);
+                        if (at < kFlips) flips[at] = (uint32_t)(k - k_lo) | ((uint32_t)tid << 16);
+                    }
                     tau[tid] = least + kGuess * job_of(tid).scale;
                     if (!split) bcur[tid] = ~0ull;
                 } else if (mine) {
@@ -1305,6 +1440,47 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         }
         }
         group_sync();
+
+        // ---- D. the syndromes and counts moved by the flips, when these are few ----
+        anew = true;
+        if constexpr (!WIDE) {
+            const int nf = keep ? (int)*n_flips : 0;
+            if (keep && nf <= few) {
+                anew = false;
+                // a warp per flip: lane j toggles its j-th check, and the old value says which way the
+                // counts of that check's symbols move; then `sg` lanes per check, one symbol each
+                uint32_t* cw = reinterpret_cast<uint32_t*>(cnt);
+                for (int q = warp; q < nf; q += nwarps) {
+                    const uint32_t what = flips[q];
+                    const int kl = (int)(what & 0xFFFFu), f = (int)(what >> 16);
+                    int mine = m;
+                    if (lane < dv_max)
+                        mine = sym_chks[4 * ((size_t)lane * sym_groups + sym_g0 + (kl >> 2)) + (kl & 3)];
+                    uint32_t was = 0u;
+                    const int bit = 2 * (f & 15);
+                    if (mine < m) was = (atomicXor(sw + 2 * mine + (f >> 4), 1u << bit) >> bit) & 1u;
+                    const int less = __popc(__ballot_sync(0xFFFFFFFFu, was != 0u));
+                    const int more = __popc(__ballot_sync(0xFFFFFFFFu, mine < m && was == 0u));
+                    if (lane == 0) atomicAdd(unsat_n + f, more - less);
+                    const int word = cnt_word(f), shift = cnt_shift(f);
+                    const uint32_t pack = ((uint32_t)mine << 1) | was;
+#pragma unroll 2
+                    for (int p = lane; p - lane < dv_max << sg_log; p += 32) {
+                        const int j = p >> sg_log;
+                        const uint32_t pj = __shfl_sync(0xFFFFFFFFu, pack, j & 31);
+                        const int i = (int)(pj >> 1);
+                        for (int e = p & ((1 << sg_log) - 1); e < dc_max && j < dv_max && i < m; e += 1 << sg_log) {
+                            const int k = chk_cols[chk_index(e, i, m)];
+                            if (k < n) {
+                                const uint32_t one = 1u << (8 * (k & 3) + shift);
+                                atomicAdd(cw + (k >> 2) * 16 + word, (pj & 1u) ? 0u - one : one);
+                            }
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        }
         ++round;
     }
 }

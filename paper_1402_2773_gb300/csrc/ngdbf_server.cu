@@ -454,7 +454,7 @@ ngdbf_status plan_serve(ngdbf_server* S, const Kind& K, ServePlan* out) {
     out->grid = sms * out->sp.bps;
     out->per_y = (size_t)pad4(K.n) * kSlots * held_bytes(K.precision);
     out->per_st = (state && !out->sp.st_smem) ? (size_t)pad4(K.n) * kSlots * 2 : 0;
-    out->bytes = align256((size_t)out->grid * out->per_y) + align256((size_t)out->grid * out->per_st);
+    out->bytes = align256((size_t)out->grid * out->per_y) + align256((size_t)out->grid * out->per_st) + kMarginSlack;
     return NGDBF_OK;
 }
 

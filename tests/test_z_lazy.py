@@ -3,6 +3,8 @@ decoder, bit for bit, where its quantization is under strain: weights, threshold
 sample ranges far apart, every symbol degree up to the 4-bit counts' limit and the bit-sliced counts
 above it, non-finite samples, and every number of live slots.
 """
+import gc
+
 import numpy as np
 import pytest
 
@@ -11,6 +13,13 @@ from paper_1402_2773_gb300 import ngdbf, workload as wl
 from test_gpu_parity import O, _gpu, assert_parity  # noqa: F401
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _collect():
+    """Tensors held by reference cycles of earlier tests go now, not while a later test counts memory."""
+    yield
+    gc.collect()
 
 
 def code_with_degree(n, m, top, seed):
