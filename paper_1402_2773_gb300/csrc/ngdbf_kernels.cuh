@@ -143,7 +143,7 @@ struct Job {
     // (rounded down), and single-bit: the lowest tau followed
     float pf_inv, pf_w, pf_bias, pf_lo, pf_hi, pf_d0, pf_d1, pf_unit, pf_rho, pf_low;
     int32_t pf_K, pf_dcap;
-    int32_t slots;              // frames a CTA takes first (1..32): the batch spread over the launch
+    int32_t slots;              // frames a CTA takes first (1..32): the batch spread over the launch (serving: 32)
     // thresholds theta lambda^u, u = 0..T: FP32 bits, binary16 values as FP32 bits, or
     // fixed-point levels Theta~(u) (FIX) or steps (FIXACC) as int32 (device memory; the
     // single-job launch passes them inline instead)
@@ -407,9 +407,6 @@ __device__ __forceinline__ int select_bit(uint32_t mask, int j) {
     }
     return pos;
 }
-
-// The first `slots` slots (1..32).
-__device__ __forceinline__ uint32_t slot_mask(int slots) { return 0xFFFFFFFFu >> (kSlots - slots); }
 
 // Lane f receives the number of lanes whose word has bit f set (a 32 x 32 bit transpose).
 __device__ __forceinline__ int column_count(uint32_t s, int lane) {
@@ -714,10 +711,13 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     constexpr bool dense = WIDE;
     // syndromes and counts kept between iterations and moved by the flips when these are few
     const bool keep = !WIDE && !split;
-    // (D: lanes per check of a flip, and the flips up to which it is used: its shared atomics, a
-    // warp instruction per 32 lanes, against the n d_v edges of A and A')
+    // D: lanes per check of a flip, 1 / dv_max (16 fraction bits), and the flips up to which it is
+    // used: their checks fit the queues' memory, and their shared atomics (about 2 lanes per cycle,
+    // d_v d_c a flip) cost less than forming all syndromes and counts: 32 flips for the (6,32) code of
+    // 2048 symbols, 63 for the (3,6) code of 1008 (16 to 64 measured alike, 128 slower by 3 to 40 %)
     const int sg_log = dc_max > 16 ? 5 : (dc_max > 1 ? 32 - __clz(dc_max - 1) : 0);
-    const int few = min(kFlips, n * dv_max / (32 * (((dv_max << sg_log) + 31) >> 5)));
+    const int dv_inv = (65536 + dv_max - 1) / dv_max;
+    const int few = min(min(kFlips, 32 * kQueue / dv_max), max(16, n / (2 << sg_log)));
     uint8_t* yb = reinterpret_cast<uint8_t*>(ys);
     uint32_t* thr = ADAPT ? reinterpret_cast<uint32_t*>(smem + L.off_thr) : nullptr;
     uint16_t* st = nullptr;
@@ -763,7 +763,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         if constexpr (CHAIN) {
             *ch.cur_e = 0;
             for (int f = 0; f < kSlots; ++f) ch.slot_e[f] = 0;     // every slot names a loaded entry
-            live = fill_chained(ch, A.chain_key, slot_mask(A.slots), 0u, 0, lane_frame, lane_start, ctl + 4);
+            live = fill_chained(ch, A.chain_key, 0xFFFFFFFFu, 0u, 0, lane_frame, lane_start, ctl + 4);
         } else {
             unsigned long long base = 0;
             const bool got = claim_frames(A, (unsigned)A.slots, &base);
@@ -1012,9 +1012,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (tid == 0 && (!split || S.rank == 0)) {
                 uint32_t fresh = 0;
                 if constexpr (CHAIN) {
-                    // (and the slots that a request admitted under a higher load allows)
-                    const uint32_t want = fin | (slot_mask(ch.jl[*ch.cur_e].slots) & ~live);
-                    fresh = fill_chained(ch, A.chain_key, want, live & ~fin, round, lane_frame, lane_start, ctl + 4);
+                    // (the finished slots and any that were left empty)
+                    fresh = fill_chained(ch, A.chain_key, ~(live & ~fin), live & ~fin, round, lane_frame, lane_start, ctl + 4);
                 } else {
                     unsigned long long base = 0;
                     const bool got = claim_frames(A, (unsigned)nfin, &base);
@@ -1168,13 +1167,13 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             const int t = round - lane_start[slot];
             const PhiloxLane ph(Jl.frame_offset + (uint64_t)lane_frame[slot], (uint32_t)t, G);
             uint32_t K = (uint32_t)Jl.pf_K, D = 0u, ebase = 0u;
-            [[maybe_unused]] int shift = 0;
+            [[maybe_unused]] uint32_t shift = 0u;        // single-bit: steps off every margin, down to 0
             if constexpr (ADAPT) {
                 const float th = (PREC == kFP32 || PREC == kFP16) ? __uint_as_float(thr[t]) : (float)(int32_t)thr[t];
                 const float d = __fmaf_rn(-Jl.pf_d1, th, Jl.pf_d0);
                 D = (uint32_t)min((int)fminf(fmaxf(d, 0.0f), 255.0f), Jl.pf_dcap) * 0x01010101u;
             } else if (single) {
-                shift = __float2int_rd(fminf(fmaxf(__fmaf_rn(-Jl.pf_d1, tau[slot], Jl.pf_d0), -255.0f), 0.0f));
+                shift = (uint32_t)-__float2int_rd(fminf(fmaxf(__fmaf_rn(-Jl.pf_d1, tau[slot], Jl.pf_d0), -255.0f), 0.0f)) * 0x01010101u;
             }
             if constexpr (CHAIN) ebase = (uint32_t)ch.slot_e[slot];
             const uint32_t csh = (uint32_t)cnt_shift(slot);
@@ -1274,12 +1273,11 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                     bool low[U][4], any = false;
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const uint32_t m4 = y4[u] + D - K * ((c4[u] >> csh) & 0x0F0F0F0Fu);
+                        uint32_t m4 = y4[u] + D - K * ((c4[u] >> csh) & 0x0F0F0F0Fu);
+                        if (single) m4 = __vsubus4(m4, shift);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            uint32_t i = __byte_perm(m4, ebase, 0x5540 + j);
-                            if (single) i = (i & ~0xFFu) | (uint32_t)max((int)(i & 0xFFu) + shift, 0);
-                            low[u][j] = r[u][j] <= cut[i];
+                            low[u][j] = r[u][j] <= cut[__byte_perm(m4, ebase, 0x5540 + j)];
                             any = any || low[u][j];
                         }
                     }
@@ -1447,34 +1445,37 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             const int nf = keep ? (int)*n_flips : 0;
             if (keep && nf <= few) {
                 anew = false;
-                // a warp per flip: lane j toggles its j-th check, and the old value says which way the
-                // counts of that check's symbols move; then `sg` lanes per check, one symbol each
-                uint32_t* cw = reinterpret_cast<uint32_t*>(cnt);
-                for (int q = warp; q < nf; q += nwarps) {
+                // a thread per (flip, check) toggles the check; the old value says which way the counts of
+                // its symbols move (kept in the queues' memory)
+                uint32_t* moves = reinterpret_cast<uint32_t*>(smem + L.off_queue);
+                const int tasks = nf * dv_max;
+                for (int i = tid; i < tasks; i += blockDim.x) {
+                    const int q = (i * dv_inv) >> 16;           // i / dv_max
                     const uint32_t what = flips[q];
-                    const int kl = (int)(what & 0xFFFFu), f = (int)(what >> 16);
-                    int mine = m;
-                    if (lane < dv_max)
-                        mine = sym_chks[4 * ((size_t)lane * sym_groups + sym_g0 + (kl >> 2)) + (kl & 3)];
-                    uint32_t was = 0u;
-                    const int bit = 2 * (f & 15);
-                    if (mine < m) was = (atomicXor(sw + 2 * mine + (f >> 4), 1u << bit) >> bit) & 1u;
-                    const int less = __popc(__ballot_sync(0xFFFFFFFFu, was != 0u));
-                    const int more = __popc(__ballot_sync(0xFFFFFFFFu, mine < m && was == 0u));
-                    if (lane == 0) atomicAdd(unsat_n + f, more - less);
-                    const int word = cnt_word(f), shift = cnt_shift(f);
-                    const uint32_t pack = ((uint32_t)mine << 1) | was;
+                    const int kl = (int)(what & 0xFFFFu), f = (int)(what >> 16), bit = 2 * (f & 15);
+                    const int c = sym_chks[4 * ((size_t)(i - q * dv_max) * sym_groups + sym_g0 + (kl >> 2)) + (kl & 3)];
+                    uint32_t move = ~0u;
+                    if (c < m) {
+                        const uint32_t was = (atomicXor(sw + 2 * c + (f >> 4), 1u << bit) >> bit) & 1u;
+                        atomicAdd(unsat_n + f, was ? -1 : 1);
+                        move = (uint32_t)c | ((uint32_t)f << 16) | (was << 21);
+                    }
+                    moves[i] = move;
+                }
+                __syncthreads();
+                // `1 << sg_log` lanes per toggled check, one of its symbols each
+                uint32_t* cw = reinterpret_cast<uint32_t*>(cnt);
+                const int per = 5 - sg_log;
 #pragma unroll 2
-                    for (int p = lane; p - lane < dv_max << sg_log; p += 32) {
-                        const int j = p >> sg_log;
-                        const uint32_t pj = __shfl_sync(0xFFFFFFFFu, pack, j & 31);
-                        const int i = (int)(pj >> 1);
-                        for (int e = p & ((1 << sg_log) - 1); e < dc_max && j < dv_max && i < m; e += 1 << sg_log) {
-                            const int k = chk_cols[chk_index(e, i, m)];
-                            if (k < n) {
-                                const uint32_t one = 1u << (8 * (k & 3) + shift);
-                                atomicAdd(cw + (k >> 2) * 16 + word, (pj & 1u) ? 0u - one : one);
-                            }
+                for (int i = (warp << per) + (lane >> sg_log); i < tasks; i += nwarps << per) {
+                    const uint32_t move = moves[i];
+                    if (move == ~0u) continue;
+                    const int c = (int)(move & 0xFFFFu), f = (int)((move >> 16) & 31u), word = cnt_word(f);
+                    for (int e = lane & ((1 << sg_log) - 1); e < dc_max; e += 1 << sg_log) {
+                        const int k = chk_cols[chk_index(e, c, m)];
+                        if (k < n) {
+                            const uint32_t one = 1u << (8 * (k & 3) + cnt_shift(f));
+                            atomicAdd(cw + (k >> 2) * 16 + word, (move >> 21) & 1u ? 0u - one : one);
                         }
                     }
                 }

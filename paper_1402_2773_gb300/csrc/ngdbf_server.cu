@@ -330,8 +330,6 @@ struct ngdbf_server {
     Kind kind;
     std::vector<Kind> seen;                  // per variant and precision: the largest layout so far
     size_t kind_scratch = 0;                 // scratch the kernel of `kind` takes at launch
-    int grid = 1;                            // its CTAs
-    int64_t frames_open = 0;                 // frames of requests submitted and not complete
     cudaEvent_t ev_kernel = nullptr;
     unsigned char* scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -354,7 +352,6 @@ void finish(ngdbf_server* S, Request* r, int32_t status) {
     r->t_done = now_s();
     r->status = status;
     S->completed.push_back(r);
-    S->frames_open -= r->job.n_frames;
     S->stats.completed += 1;
     if (status != NGDBF_OK) S->stats.failed += 1;
     else S->stats.frames += r->job.n_frames;
@@ -390,8 +387,6 @@ ngdbf_status admit(ngdbf_server* S, Request* r) {
              sg.thr);
     r->dj.thr = dthr;
     r->dj.gen = r->gen;
-    // the unfinished requests' frames spread over the resident CTAs
-    r->dj.slots = first_slots(S->frames_open, S->grid);
     // requests of the same code and parameters share a chain key: the kernel decodes frames
     // of several of them in one CTA's slots (they differ only in samples, sigma, offset, outputs)
     {
@@ -624,7 +619,6 @@ void scheduler(ngdbf_server* S) {
                     continue;
                 }
                 S->kind_scratch = P.bytes;
-                S->grid = P.grid;
             }
             const size_t reserve = S->running ? 0 : S->kind_scratch;   // scratch of a kernel still to be launched
             if (S->in_use + reserve + bytes > S->budget) {
@@ -775,7 +769,6 @@ extern "C" ngdbf_status ngdbf_server_submit(ngdbf_server_t* S, const ngdbf_code_
         std::lock_guard<std::mutex> lk(S->mu);
         r->id = ++S->stats.submitted;
         r->t_submit = now_s();
-        S->frames_open += r->job.n_frames;
         S->pending.push_back(r);
     }
     S->cv.notify_all();
