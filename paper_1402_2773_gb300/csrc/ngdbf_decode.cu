@@ -819,9 +819,10 @@ ngdbf_status ngdbf_decode_host(const ngdbf_code_t* C, const float* y_host, int64
     if (!y_host || !bits_host || !iters_host || !pass_host) return fail(NGDBF_ERR_INVALID_ARG, "NULL buffer");
     const int64_t n = C->n, nb = (C->n + 7) / 8;
     // chunk sizes: the caller's, or a ramp -- an eighth of a quarter of the call first (so
-    // that little copying is exposed before the first decode), doubling up to a quarter of
-    // the call (so that only the last chunk's tail, where a CTA waits for its slowest frame,
-    // is exposed), chunks between 256 MB and 2 GB of samples and at least 4096 frames
+    // that little copying is exposed before the first decode), then four times the last (a
+    // chunk decodes in four times its copy and more) up to a quarter of the call (so that only
+    // the last chunk's tail, where a CTA waits for its slowest frame, is exposed), chunks
+    // between 256 MB and 2 GB of samples and at least 4096 frames
     int64_t first_chunk = chunk_frames;
     if (chunk_frames <= 0) {
         const int64_t lo = std::max<int64_t>(4096, (int64_t)(256ll << 20) / (4 * n));
@@ -867,7 +868,7 @@ ngdbf_status ngdbf_decode_host(const ngdbf_code_t* C, const float* y_host, int64
     Staging* stage = host_copy_mode() == NGDBF_HOST_COPY_STAGED ? staging_acquire(dev) : nullptr;
     int64_t kernels = 0, chunks = 0;
     for (int64_t off = 0, c = 0, size = first_chunk; off < n_frames && rs == NGDBF_OK;
-         off += size, size = std::min(2 * size, chunk_frames), ++c) {
+         off += size, size = std::min(4 * size, chunk_frames), ++c) {
         const int b = (int)(c & 1);
         const int64_t F = std::min(size, n_frames - off);
         unsigned char* p = static_cast<unsigned char*>(buf[b]);
