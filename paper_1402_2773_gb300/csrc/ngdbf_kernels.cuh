@@ -1289,14 +1289,17 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                             if (!(act && step + u < s_end && gl + u * stride < groups_l)) mark[u] = 0u;
                         }
                         if (ALL || each > 2) {
-#pragma unroll 1
-                            for (int u = 0; u < U; ++u) {
-                                const uint32_t mk = u ? mark[U - 1] : mark[0];
-                                const uint32_t b = __ballot_sync(0xFFFFFFFFu, mk != 0u);
-                                if (mk)
-                                    queue[queued + __popc(b & ((1u << lane) - 1u))] =
-                                        (uint32_t)(gl + u * stride) | ((uint32_t)slot << 16) | (mk << 24);
-                                queued += __popc(b);
+                            uint32_t b[U];
+#pragma unroll
+                            for (int u = 0; u < U; ++u) b[u] = __ballot_sync(0xFFFFFFFFu, mark[u] != 0u);
+                            const uint32_t lt = (1u << lane) - 1u;
+                            const uint32_t what = (uint32_t)gl | ((uint32_t)slot << 16);
+                            if (mark[0]) queue[queued + __popc(b[0] & lt)] = what | (mark[0] << 24);
+                            queued += __popc(b[0]);
+                            while (queued >= 32) evaluate(32);
+                            if constexpr (U > 1) {
+                                if (mark[U - 1]) queue[queued + __popc(b[U - 1] & lt)] = (what + stride) | (mark[U - 1] << 24);
+                                queued += __popc(b[U - 1]);
                                 while (queued >= 32) evaluate(32);
                             }
                         } else {
