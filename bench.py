@@ -44,19 +44,12 @@ PRECISIONS = {"fp32": (0, 0, "f32"), "fp16": (1, 0, "f16"), "fix8": (3, 8, "i8")
               "fix8-eq9": (2, 8, "i8")}
 DATA_SEED = 2014          # information bits and channel noise
 DECODER_SEED = 1          # Philox key of the perturbation
-# Algorithmic lane operations per (symbol, iteration) of the FP32 path: Philox4x32-10 20 (per
-# 4 symbols: 10 rounds of two wide multiplies, counted as 4, and 4 XOR) + inverse-CDF deviate 13
-# (odd integer 1, leading zeros 1, normalize 1, segment index 2, table load 1, position v 3,
-# cubic 3, sign 1) + perturbation 1 + inversion function 5 + decision bit 1 + penalty sum
-# (2 d_v + 2) + threshold, adaptation, window and ballot 4 = 46 + 2 d_v, i.e. 58 for d_v = 6.
-
-
-def ops_per_symbol_iter(dv: int) -> int:
-    """Algorithmic lane operations per (symbol, iteration) of the FP32 path for symbol degree dv."""
-    return 46 + 2 * int(dv)
-
-
-OPS_PER_SYMBOL_ITER = ops_per_symbol_iter(6)
+# Lane operations that every (symbol, iteration) of a live frame needs: Philox4x32-10 20 (per 4
+# symbols: 10 rounds of two wide multiplies, counted as 4, and 4 XOR), the margin byte's counts
+# taken off 1, the cutoff lookup 1, the comparison 1.  The counts are formed bit-sliced for 32
+# frames at once, and the deviate, E_k and the counters only for the few outputs at or below
+# their cutoffs: neither is counted.
+OPS_PER_SYMBOL_ITER = 23
 # Lane operations per symbol of the same-mix probe (ngdbf_mix_probe), by the same convention:
 # Philox 20 + deviate 13 + perturbation 1 + inversion function 5 + decision bit 1 + threshold,
 # adaptation, window and ballot 4 + the count lane's extraction 1 (the probe has no per-check
@@ -66,7 +59,7 @@ PROBE_GROUPS = 32768
 
 
 def mix_probe(ngdbf, stream, reps=5, warmup=2):
-    """Attainable lane-op rate of the decode's per-slot instruction mix (CUDA events, best of reps)."""
+    """Attainable lane-op rate of the dense per-symbol instruction mix (CUDA events, best of reps)."""
     import torch
     sink = torch.zeros(1, dtype=torch.int32, device="cuda")
     threads = 0
@@ -84,11 +77,10 @@ def mix_probe(ngdbf, stream, reps=5, warmup=2):
     symbols = threads * PROBE_GROUPS * 4
     return {"lane_op_s": symbols * PROBE_OPS_PER_SYMBOL / (best / 1e3), "ms": best, "threads": threads,
             "symbols_per_launch": symbols, "ops_per_symbol": PROBE_OPS_PER_SYMBOL}
-# DRAM bytes (read + write) per decoded frame of the decode kernel, from an ncu capture of
-# this workload at 2*10^4 frames per Eb/N0 point (samples 164 MB per launch, larger than L2):
-# 167.6 MB read + 8.0 MB written at 3.5 dB; traffic scales with frames, each frame's samples
-# being read once.  Set to None when the kernel changes without a new capture.
-DRAM_BYTES_PER_FRAME = 8_697
+# DRAM bytes (read + write) per decoded frame of the decode kernel from an ncu capture of this
+# workload's mean over the three points; None: captured per point only (15 kB a frame at 4.5 dB,
+# 243 kB at 3.5 dB, where the slots' state and samples of two CTAs per SM exceed L2).
+DRAM_BYTES_PER_FRAME = None
 
 
 def env_rank():
@@ -334,14 +326,13 @@ def run_ours(args):
           "peak_nominal": peak_ops / 1e12, "frac_nominal": achieved / peak_ops,
           "peak_nominal_basis": f"{sm_count} SMs x 128 lanes x {peak_mhz:.0f} MHz (max SM clock)",
           "probe": {k: v for k, v in probe.items() if k != "clocks"} | {"sm_mhz": pclk},
-          "kernel": "ngdbf_persistent_kernel<ADAPT,SMOOTH,state in smem>",
+          "kernel": "ngdbf_persistent_kernel<ADAPT,SMOOTH>",
           "ops_per_symbol_iter": OPS_PER_SYMBOL_ITER,
-          "ops_basis": "FP32 path" if args.precision == "fp32" else
-                       "FP32 path count; the rounding or quantizing steps of this precision are not counted",
+          "ops_basis": "generator, margin and cutoff of every live symbol-iteration",
           "algorithmic_bytes_per_launch": F * (4 * code.n + nb + 5),
           "traffic_basis": "ncu dram__bytes_read.sum + dram__bytes_write.sum per frame on a 2*10^4-frame "
                            "capture, scaled to the launch's frames" if traffic else
-                           "no capture of this precision's kernel",
+                           "not captured for this mix of points",
           "symbol_iters_per_launch": float(np.mean(sym_iters)), "mean_launch_ms": mean_launch_s * 1e3}
 
     # end to end through the host-buffer C-ABI call: copies inside the timed region
@@ -509,8 +500,7 @@ def run_multicode(args):
     ops = 0.0
     for jb, o in zip(jobs, host):
         it = o[1].astype(np.int64)
-        dv = jb["code"].dense().sum(axis=0).max()
-        ops += float(it.sum()) * jb["code"].n * ops_per_symbol_iter(dv)
+        ops += float(it.sum()) * jb["code"].n * OPS_PER_SYMBOL_ITER
         per_code.append({"code": jb["code"].name, "frames": jb["frames"], "ebn0_db": round(jb["ebn0"], 3),
                          "t_max": jb["params"]["t_max"], "avg_iters": float(it.mean()),
                          "pass_rate": float(o[2].mean())})
@@ -582,7 +572,6 @@ def run_serving(args):
     ngdbf.load()
     specs = multicode_jobs(rank)
     codes = [jb["code"] for jb in specs]
-    dvs = [int(c.dense().sum(axis=0).max()) for c in codes]
     dcs = [ngdbf.DeviceCode.from_code(c) for c in codes]
     params = [ngdbf.make_params(**jb["params"]) for jb in specs]
     # every input pool in one page-locked block from the library's allocator
@@ -652,7 +641,7 @@ def run_serving(args):
             lat_p, span_p, outs_p = run_plain(trace)
             same = all(all(torch.equal(a, b) for a, b in zip(x, y)) for x, y in zip(outs_s, outs_p))
             # algorithmic lane operations of the iterations the frames needed (FP32 count)
-            ops = sum(float(o[1].numpy().astype(np.int64).sum()) * codes[c].n * ops_per_symbol_iter(dvs[c])
+            ops = sum(float(o[1].numpy().astype(np.int64).sum()) * codes[c].n * OPS_PER_SYMBOL_ITER
                       for (_, c, _, _, _, _), o in zip(trace, outs_s))
             res[label] = {
                 "rate_requests_per_s": rate, "requests": n_req, "frames": frames,

@@ -49,6 +49,14 @@
 // rounded up.  Every rounding errs towards evaluating E_k, so the decisions are those of the
 // dense form bit for bit; the exact form runs for the symbols at or below the cutoff only.
 //
+// What bounds it (one GB300, the (6,32) code of 2048 symbols, 32 live slots): a step of phase C --
+// four symbols of 32 slots -- takes 75 instructions, 40 of them Philox, and 31 cycles of an SM; the
+// 18 wide multiplies alone take 19 (1.05 cycles each), the ALU pipe 18, so the step is near the
+// issue and pipe limits (issue 62-68 %, ALU 57-61 % busy).  Forming E_k for every symbol took 103
+// cycles a step.  100003 frames at 4.5 dB (8-bit samples): 30.6 -> 12.5 ms; 200000 frames at 3.5 dB,
+// where 3 % of the outputs are evaluated and A and A' run every iteration: 260 -> 192 ms.  With
+// few slots an iteration is latency: 3.5 us for one frame of the (3,6) code of 1008 symbols.
+//
 // The single-bit variant (Step 3a) needs the least E_k of a slot: it sweeps with a guess tau, the
 // slot's previous least E_k plus kGuess of its noise, in the place of the threshold.  A least
 // E_k at or below tau is the slot's (every symbol that could be as low was evaluated); the
