@@ -150,13 +150,14 @@ ngdbf_status ngdbf_code_info(const ngdbf_code_t* code, int32_t* n, int32_t* m,
  *   pass         DEVICE uint8[n_frames] (written)
  *   stream       cudaStream_t to run on (NULL = legacy default stream)
  * Asynchronous: returns after enqueueing; outputs are valid once the stream
- * reaches this point.  Temporary device memory (per-slot sample copies and
- * a work counter, about 160 * n bytes per 32 concurrently decoded frames)
- * is taken from a library-owned stream-ordered pool and returned on the
- * same stream.  All pointers must be device memory of the current device.
+ * reaches this point; y must stay unchanged until then (it is read while
+ * frames are decoded).  Temporary device memory (per-slot margins, for large
+ * batches and long codes the per-slot state, and a work counter: 32 to 96 * n
+ * bytes per resident CTA) is taken from a library-owned stream-ordered pool
+ * and returned on the same stream.  All pointers must be device memory of the current device.
  * The decision, syndrome and count words of one CTA's 32 frames must fit the
- * device's shared memory per block (about 20 n + 16 m + 5 KB bytes for symbol
- * degrees up to 7: n up to about 8,000 at rate 1/2 on a 227 KB device); larger
+ * device's shared memory per block (about 20 n + 8 m + 7 KB bytes for symbol
+ * degrees up to 15: n up to about 9,300 at rate 1/2 on a 227 KB device); larger
  * codes are rejected with NGDBF_ERR_UNSUPPORTED.
  * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA.
  */
@@ -211,7 +212,7 @@ ngdbf_status ngdbf_decode_plain(const ngdbf_code_t* code, const float* y, int64_
  * Outputs are copied straight into the caller's buffers.  Same layouts as
  * ngdbf_decode.
  * chunk_frames <= 0 picks chunk sizes automatically: a quarter of the call
- * (between 256 MB and 2 GB of samples, at least 4096 frames), reached by doubling
+ * (between 256 MB and 2 GB of samples, at least 4096 frames), reached in steps of four
  * from an eighth of it so that little copying precedes the first decode; two
  * chunks of device scratch are held at a time.
  */

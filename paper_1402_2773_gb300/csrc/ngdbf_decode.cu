@@ -73,9 +73,9 @@ template <bool ADAPT, bool SMOOTH, bool ST_SMEM, bool WIDE, int PREC>
 __global__ void __launch_bounds__(1024) ngdbf_persistent_kernel(const __grid_constant__ DecodeArgs A) {
     using HeldT = typename Held<PREC>::T;
     const Job& J = A.J;
-    HeldT* ys = static_cast<HeldT*>(A.yslots) + (size_t)blockIdx.x * pad4(J.n) * kSlots;
+    HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, J.n);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(J.n) * kSlots : nullptr;
-    decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, with_fixed_offsets(A.L), A.placement, ys, st);
+    decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, with_fixed_offsets<WIDE>(A.L), A.placement, ys, st);
 }
 
 }  // namespace ngdbf
@@ -110,7 +110,7 @@ void set_last_launch(int grid, int block, int smem, int state_in_smem, int table
     g_last_launch.state_in_smem = state_in_smem;
     g_last_launch.kernels = kernels;
     g_last_launch.sm_count = sm_count;
-    g_last_launch.tables_in_smem = tables_in_smem;
+    g_last_launch.tables_in_smem = tables_in_smem & (kTabChk | kTabSym);
 }
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -259,6 +259,9 @@ KernelFn pick_kernel(int variant, int precision, bool st_smem, bool wide) {
     }
 }
 
+// Bytes of slot scratch per (symbol, slot): the margin byte, or the held sample of wide codes.
+size_t slot_bytes(int precision, bool wide) { return wide ? held_bytes(precision) : 1; }
+
 // Bytes of one held sample.
 size_t held_bytes(int precision) {
     return precision == NGDBF_FP16 ? 2 : ((precision == NGDBF_FIX || precision == NGDBF_FIXACC) ? 1 : 4);
@@ -306,10 +309,12 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
         // CTAs of 512 threads or more share an SM
         if (best.bps > 0 && !(many && best.bps == 1)) break;
         const bool second = best.bps > 0;
-        for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
+        for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0, kTight}) {
+            if (tb == kTight && (best.bps > 0 || st || dv_max > kNarrowDegree)) continue;    // only where nothing else fits
             const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, n_local);
             if (L.total > limit) continue;
-            for (const int block : {1024, 512, 256}) {
+            for (const int block : {1024, 512, 256, kTightThreads}) {
+                if ((tb == kTight) != (block == kTightThreads)) continue;
                 int bps = 0;
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, block, L.total);
                 if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
@@ -608,12 +613,23 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     s = get_pool(dev, &pool);
     if (s != NGDBF_OK) return s;
     const bool state = (P->variant & 3) != 0;
-    const size_t slot_elems = (size_t)plan.grid * pad4(C->n) * kSlots;
-    const size_t bytes_y = (slot_elems * held_bytes(P->precision) + 255) / 256 * 256;
-    const size_t bytes_st = (state && !plan.st_smem) ? (slot_elems * 2 + 255) / 256 * 256 : 0;
-    const size_t total = 256 + bytes_y + bytes_st + kMarginSlack;
+    size_t bytes_y = 0, bytes_st = 0;
     void* ws = nullptr;
-    e = cudaMallocFromPoolAsync(&ws, total, pool, stream);
+    auto take_scratch = [&]() {
+        const size_t slot_elems = (size_t)plan.grid * pad4(C->n) * kSlots;
+        bytes_y = align256(slot_elems * slot_bytes(P->precision, C->dv_max > kNarrowDegree));
+        bytes_st = (state && !plan.st_smem) ? align256(slot_elems * 2) : 0;
+        return cudaMallocFromPoolAsync(&ws, 256 + bytes_y + bytes_st + kMarginSlack, pool, stream);
+    };
+    e = take_scratch();
+    if (e == cudaErrorMemoryAllocation) {
+        // as little scratch as 32 frames to a CTA need, one CTA per SM
+        cudaGetLastError();
+        s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count, true);
+        if (s != NGDBF_OK) return s;
+        plan.grid = (int)std::min<int64_t>(plan.grid, (n_frames + kSlots - 1) / kSlots);
+        e = take_scratch();
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(e == cudaErrorMemoryAllocation ? NGDBF_ERR_OOM : NGDBF_ERR_CUDA,
@@ -1106,15 +1122,17 @@ std::vector<int32_t> assign_ctas_capped(const std::vector<int64_t>& frames, cons
 // of the `tables` as fit in `limit`; -1 when some job does not fit at all.  With a cluster of
 // C > 1 CTAs, jobs of at least split_min_n symbols hold their share of the symbols per CTA.
 int table_smem(const ngdbf_job* jobs, int32_t n_jobs, int C, int split_min_n, bool adapt, bool st, bool wide,
-               int tables, int limit) {
+               int tables, int limit, bool* tight = nullptr) {
     int total = 0;
+    if (tight) *tight = false;
     for (int j = 0; j < n_jobs; ++j) {
         const ngdbf_code* c = jobs[j].code;
         const int n_local = (C > 1 && c->n >= split_min_n) ? split_local_max(c->n, C) : c->n;
         int tb = 0;
         const SmemLayout L = job_layout(c->n, c->m, jobs[j].params.t_max, c->dv_max, c->dc_max, adapt, st, wide,
                                         tables, n_local, limit, &tb);
-        if (L.total > limit) return -1;
+        if (L.total > limit || ((tb & kTight) && !tight)) return -1;
+        if (tb & kTight) *tight = true;
         total = std::max(total, L.total);
     }
     return total;
@@ -1163,9 +1181,11 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
-            const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, st, T.wide, tb, limit);
+            bool tight = false;         // some job needs the tight layout: its block size for all
+            const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, st, T.wide, tb, limit, &tight);
             if (total < 0) continue;
-            for (const int block : {1024, 512, 256}) {
+            for (const int block : {1024, 512, 256, kTightThreads}) {
+                if (tight != (block == kTightThreads)) continue;
                 int bps = 0;
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)fn, block, total);
                 if (e != cudaSuccess) return cuda_fail(e, "occupancy");
@@ -1177,13 +1197,15 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
                     T.smem = total;
                     T.st_smem = st;
                     T.placement = tb;
+                    T.tight = tight;
                 }
             }
         }
     }
     if (best_bps == 0) return fail(NGDBF_ERR_UNSUPPORTED, "code too large for the shared-memory decision words");
     T.state_global = state && !T.st_smem;
-    for (int block : {1024, 512, 256}) {
+    for (int block : {1024, 512, 256, kTightThreads}) {
+        if (T.tight != (block == kTightThreads)) continue;
         int bps = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)T.fn, block, T.smem);
         if (e != cudaSuccess) return cuda_fail(e, "occupancy");
@@ -1414,7 +1436,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     size_t grid_max = 0, bytes_y = 0, bytes_st = 0;
     for (const TableShape& sh : B->shapes) {
         grid_max = std::max(grid_max, (size_t)sh.grid_max);
-        bytes_y = std::max(bytes_y, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * held_bytes(T.precision));
+        bytes_y = std::max(bytes_y, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * slot_bytes(T.precision, T.wide));
         if (sh.state_global) bytes_st = std::max(bytes_st, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * 2);
     }
     const size_t off_jobs = 0, off_thr = align256(sizeof(Job) * n_jobs), off_q = off_thr + align256(T.thr_words * 4);

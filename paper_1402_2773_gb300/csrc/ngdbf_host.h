@@ -36,8 +36,9 @@ size_t align256(size_t v);
 ngdbf_status get_pool(int dev, cudaMemPool_t* out);
 // Philox round keys and series coefficients of the perturbation generator.
 void host_gen_consts(uint64_t seed, GenConsts& G);
-// Bytes of one held sample of a precision.
+// Bytes of one held sample of a precision; of slot scratch per (symbol, slot).
 size_t held_bytes(int precision);
+size_t slot_bytes(int precision, bool wide);
 ngdbf_status check_params(const ngdbf_params* P, float sigma);
 // Shared-memory plan of a kernel of the slot loop for the given maxima: per-slot state in
 // shared memory when it fits (fn_st) else global (fn_nost), adjacency tables, block size.
@@ -58,6 +59,7 @@ struct TablePlan {
     int n_max = 0, m_max = 0, t_max = 0, dv_max = 0, dc_max = 0;
     int variant = 0, precision = 0, sm_count = 0, smem = 0;
     bool st_smem = false, wide = false, state_global = false;
+    bool tight = false;         // some job is laid out with kTight: blocks of kTightThreads
     int placement = 0;          // adjacency tables in shared memory: kTabChk | kTabSym
     size_t thr_words = 0;
     void* fn = nullptr;

@@ -90,6 +90,11 @@ __host__ __device__ inline int chk_entries(int m, int dc_max) { return m * 8 * (
 __host__ __device__ inline int gidx(int k, int f) { return (((k >> 2) * kSlots + f) << 2) | (k & 3); }
 constexpr int kTabChk = 1;              // N(i) table in shared memory
 constexpr int kTabSym = 2;              // M(k) table and degrees in shared memory
+// The longest codes (without their state in shared memory, and at most kTightThreads threads): the
+// warps' queues lie over the syndrome words, which phase C does not read, and flips are not
+// recorded (no D).  Every check has at most 64 symbols, so there are words enough.
+constexpr int kTight = 4;
+constexpr int kTightThreads = 128;
 
 constexpr int kMaxT = NGDBF_MAX_T;
 constexpr uint32_t kUMask = 0x1FFu;   // flips of the symbol so far: bits 0-8
@@ -120,6 +125,15 @@ template <> struct Held<kFP32> { using T = float; };
 template <> struct Held<kFP16> { using T = __half; };
 template <> struct Held<kFIX> { using T = int8_t; };      // signed level code b, value 2b + 1
 template <> struct Held<kFIXACC> { using T = int8_t; };   // the same Eq. 8 level code
+
+// Bytes of slot scratch per (symbol, slot): the margin byte, or with bit-sliced counts (wide) the
+// held sample; and the scratch of CTA `cta` of a launch whose CTAs hold n symbols each.
+template <int PREC, bool WIDE>
+__device__ __forceinline__ typename Held<PREC>::T* slot_scratch(void* base, int cta, int n) {
+    using T = typename Held<PREC>::T;
+    const size_t at = (size_t)cta * pad4(n) * kSlots;
+    return WIDE ? static_cast<T*>(base) + at : reinterpret_cast<T*>(static_cast<uint8_t*>(base) + at);
+}
 
 // One decode job: a code, a batch of frames and the parameters of the method.
 struct Job {
@@ -231,7 +245,7 @@ struct SmemLayout {
 struct DecodeArgs {
     Job J;
     int32_t placement;          // adjacency tables copied into shared memory: kTabChk | kTabSym
-    void* yslots;               // [grid][pad4(n)/4][32][4] held samples (4, 2 or 1 bytes each)
+    void* yslots;               // [grid][pad4(n)/4][32][4] margin bytes (wide: held samples of 4, 2 or 1 bytes)
     uint16_t* st_global;        // [grid][pad4(n)/4][32][4] when the state is not in shared memory
     SmemLayout L;
     GenConsts G;
@@ -308,19 +322,22 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     L.off_frame = take(kSlots * 8, 16);
     L.off_start = take(kSlots * 4, 16);
     L.off_ctl = take(8 * 4, 16);
-    L.off_unsat = take(kSlots * 4, 16);    // number of unsatisfied checks of each slot
-    L.off_flips = take(kFlips * 4, 16);    // flips of this iteration: local symbol | slot << 16
+    const bool tight = (tables & kTight) != 0;
+    // (wide: none of the lazy form's arrays)
+    L.off_unsat = wd ? -1 : take(kSlots * 4, 16);   // number of unsatisfied checks of each slot
     L.off_best = take(2 * kSlots * 8, 16); // single-bit variant: least (E key, k) per slot, two rounds
-    L.off_tau = take(kSlots * 4, 16);      // single-bit variant: guess of each slot's least E_k
+    L.off_tau = wd ? -1 : take(kSlots * 4, 16);     // single-bit variant: guess of each slot's least E_k
     L.off_trace = take(kSlots * 12, 16);   // objective trace: per slot C (int64), then U (int32)
     L.off_icdf = take(256 * 16, 16);       // inverse normal CDF coefficients
-    L.off_cut = take(256 * 4, 16);         // cutoff of each margin byte
+    L.off_cut = wd ? -1 : take(256 * 4, 16);        // cutoff of each margin byte
     L.off_cnt = take(pad4(n_local) * cnt_bytes, 16);
+    L.off_flips = wd || tight ? -1 : take(kFlips * 4, 16);   // flips of this iteration: local symbol | slot << 16
     // per warp: groups for the exact form (phase C's last steps may read up to 31 groups of counts
     // past the code's: they lie inside this array)
-    L.off_queue = take(32 * kQueue * 4, 16);
+    L.off_queue = wd || tight ? -1 : take(32 * kQueue * 4, 16);
     L.off_xw = take(pad4(n + 1) * 4, 16);
     L.off_sw = take((m + 1) * (wd ? 4 : 8), 16);
+    if (tight) L.off_queue = L.off_sw;
     // all 512 values of the 9-bit u field: an idle slot's counter may pass T (its lookups are
     // don't-care but stay inside the table)
     L.off_thr = need_thr ? take((kUMask + 1) * 4, 16) : -1;
@@ -331,15 +348,15 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     return L;
 }
 
-// Layout L with the offsets that do not depend on the code (all up to the counts) as compile-time
-// constants.
+// Layout L of a narrow or wide kernel with the offsets that do not depend on the code (all up to
+// the counts) as compile-time constants.
+template <bool WIDE>
 __device__ __forceinline__ SmemLayout with_fixed_offsets(SmemLayout L) {
-    const SmemLayout F = smem_layout(4, 1, 0, 1, 1, false, false, 0);
+    const SmemLayout F = smem_layout(4, 1, 0, 1, 1, false, false, 0, -1, WIDE ? 1 : 0);
     L.off_frame = F.off_frame;
     L.off_start = F.off_start;
     L.off_ctl = F.off_ctl;
     L.off_unsat = F.off_unsat;
-    L.off_flips = F.off_flips;
     L.off_best = F.off_best;
     L.off_tau = F.off_tau;
     L.off_trace = F.off_trace;
@@ -352,15 +369,15 @@ __device__ __forceinline__ SmemLayout with_fixed_offsets(SmemLayout L) {
 // Layout of one job of a job table: arrays sized for the job's own code (n_local symbols per
 // CTA: its share when split over a cluster) in the launch's count and syndrome format, with
 // as many of the adjacency tables that `tables` allows as fit in `bytes` (both, then N(i)
-// alone, M(k) alone, none); *tables_out receives the placement taken.  Host planning and the kernel
+// alone, M(k) alone, none, then kTight without state); *tables_out receives the placement taken.  Host planning and the kernel
 // evaluate it alike, so the launch's shared memory is the largest job's, not the layout of
 // the table's maxima.
 __host__ __device__ inline SmemLayout job_layout(int n, int m, int t_max, int dv_max, int dc_max, bool need_thr,
                                                  bool st_smem, bool wide, int tables, int n_local, int bytes,
                                                  int* tables_out) {
-    const int opts[4] = {tables & (kTabChk | kTabSym), tables & kTabChk, tables & kTabSym, 0};
+    const int opts[5] = {tables & (kTabChk | kTabSym), tables & kTabChk, tables & kTabSym, 0, kTight};
     SmemLayout L{};
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < (wide || st_smem ? 4 : 5); ++i) {
         L = smem_layout(n, m, t_max, dv_max, dc_max, need_thr, st_smem, opts[i], n_local, wide ? 1 : 0);
         *tables_out = opts[i];
         if (L.total <= bytes) break;
@@ -726,6 +743,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     const int sg_log = dc_max > 16 ? 5 : (dc_max > 1 ? 32 - __clz(dc_max - 1) : 0);
     const int dv_inv = (65536 + dv_max - 1) / dv_max;
     const int few = min(min(kFlips, 32 * kQueue / dv_max), max(16, n / (2 << sg_log)));
+    const bool record = keep && (tables & kTight) == 0;
     uint8_t* yb = reinterpret_cast<uint8_t*>(ys);
     uint32_t* thr = ADAPT ? reinterpret_cast<uint32_t*>(smem + L.off_thr) : nullptr;
     uint16_t* st = nullptr;
@@ -799,7 +817,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     for (int k = tid; k < pad4(n + 1); k += blockDim.x) xw[k] = 0u;
     for (int i = tid; i < (m + 1) * (WIDE ? 1 : 2); i += blockDim.x) sw[i] = 0u;
     // (an unsplit chaining CTA makes entry 0's table here, the others' when they are loaded)
-    for (int i = tid; i < 256; i += blockDim.x) cut[i] = margin_cutoff(i, A);
+    if constexpr (!WIDE)
+        for (int i = tid; i < 256; i += blockDim.x) cut[i] = margin_cutoff(i, A);
     // the missing symbols of a partial last group: margins that nothing undercuts
     if (!dense)
         for (int e = nl * kSlots + tid; e < pad4(nl) * kSlots; e += blockDim.x)
@@ -844,7 +863,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             // ---- load new frames: saturated samples into the slot columns, x(0) = sign(y) ----
             // (four samples in flight per thread)
             const uint32_t fresh = ctl[3];
-            if (single && tid < kSlots && ((fresh >> tid) & 1u)) tau[tid] = A.pf_low + kFirst * job_of(tid).scale;
+            if (!dense && single && tid < kSlots && ((fresh >> tid) & 1u)) tau[tid] = A.pf_low + kFirst * job_of(tid).scale;
             if constexpr (CHAIN) {
                 for (uint32_t r = ctl[4]; r; r &= r - 1) {
                     const int e = __ffs(r) - 1;
@@ -1226,7 +1245,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 }
                 // recorded while they are few enough to be used (D)
                 const uint32_t fl = __ballot_sync(0xFFFFFFFFu, flip);
-                if (fl && keep && *(volatile uint32_t*)n_flips <= (uint32_t)few) {
+                if (fl && record && *(volatile uint32_t*)n_flips <= (uint32_t)few) {
                     int at = 0;
                     if (lane == 0) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
                     at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(fl & ((1u << lane) - 1u));
@@ -1428,13 +1447,13 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                                                                 was_neg ? 0u : 0x80000000u, sym_deg[k - sym_base], Jf);
                         }
                     }
-                    if (keep) {
+                    if (record) {
                         const int at = (int)atomicAdd(n_flips, 1u);
                         if (at < kFlips) flips[at] = (uint32_t)(k - k_lo) | ((uint32_t)tid << 16);
                     }
-                    tau[tid] = least + kGuess * job_of(tid).scale;
+                    if constexpr (!dense) tau[tid] = least + kGuess * job_of(tid).scale;
                     if (!split) bcur[tid] = ~0ull;
-                } else if (mine) {
+                } else if (!dense && mine) {
                     tau[tid] = sweep < kSweeps ? tau[tid] + kRaise * job_of(tid).scale : INFINITY;
                 }
                 // when split, the buffer of the next round (the other CTAs finished reading it
@@ -1453,8 +1472,8 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         // ---- D. the syndromes and counts moved by the flips, when these are few ----
         anew = true;
         if constexpr (!WIDE) {
-            const int nf = keep ? (int)*n_flips : 0;
-            if (keep && nf <= few) {
+            const int nf = record ? (int)*n_flips : 0;
+            if (record && nf <= few) {
                 anew = false;
                 // a thread per (flip, check) toggles the check; the old value says which way the counts of
                 // its symbols move (kept in the queues' memory)

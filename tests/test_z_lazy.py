@@ -88,3 +88,14 @@ def test_live_slots(O, F, variant):
     code = wl.code_from_dense(wl.peg_code(512, 256, 3, seed=2).dense()[:, :509])
     y, _, sig = wl.frames(code, F, 2.5, seed=F)
     assert_parity(O, code, y, sig, seed=1, frame_offset=2 ** 32 - 7, variant=variant, lam=0.97, t_max=60, smooth_window=10)
+
+
+@pytest.mark.parametrize("variant", [0, 3, 4])
+def test_longest_codes(O, variant):
+    """A code whose arrays fit shared memory only with the queues over the syndrome words."""
+    n, m = 10950, 300
+    H = np.zeros((m, n), np.uint8)
+    H[np.arange(n) % m, np.arange(n)] = 1
+    code = wl.code_from_dense(H)
+    y, _, _ = wl.frames(code, 40, None, seed=5, sigma=0.8)
+    assert_parity(O, code, y, 0.8, seed=2, variant=variant, lam=0.95, t_max=8, smooth_window=3, w=0.4, theta=-0.5)
