@@ -78,8 +78,8 @@ def mix_probe(ngdbf, stream, reps=5, warmup=2):
     return {"lane_op_s": symbols * PROBE_OPS_PER_SYMBOL / (best / 1e3), "ms": best, "threads": threads,
             "symbols_per_launch": symbols, "ops_per_symbol": PROBE_OPS_PER_SYMBOL}
 # DRAM bytes (read + write) per decoded frame of the decode kernel from an ncu capture of this
-# workload's mean over the three points; None: captured per point only (15 kB a frame at 4.5 dB,
-# 243 kB at 3.5 dB, where the slots' state and samples of two CTAs per SM exceed L2).
+# workload's mean over the three points; None: captured per point only (13 kB a frame at 4.5 dB,
+# 178 kB at 3.5 dB, where the slots' state and samples of two CTAs per SM exceed L2).
 DRAM_BYTES_PER_FRAME = None
 
 
