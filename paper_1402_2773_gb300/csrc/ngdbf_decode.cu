@@ -444,7 +444,10 @@ void fill_margins(const ngdbf_code* C, const ngdbf_params* P, const uint32_t* th
     const double ymag = J.clamp ? 1.001 * J.y_max : 300.0 * step;
     const double mag = 2.0 * (std::fabs(hi * unit) + ymag) + 4.0 * w * d + 16.0 * scale;
     double slack = std::ldexp(mag, -21);
-    if (P->precision == NGDBF_FP16) slack = std::ldexp(2.0 * ymag + 4.0 * w * d + 16.0 * scale, -11) + 1e-6;
+    // (binary16: an E_k near a threshold above zero is as large as it, whatever the samples' range;
+    // near one below zero its terms are no larger than the weights and the noise)
+    if (P->precision == NGDBF_FP16)
+        slack = std::ldexp(2.0 * (std::max(hi, 0.0) + ymag) + 4.0 * w * d + 16.0 * scale, -11) + 1e-6;
     else if (P->precision == NGDBF_FIX) slack += 1.001 * unit;
     else if (P->precision == NGDBF_FIXACC) slack += 0.501 * unit;
     const double round = 0.02 + std::ldexp(std::fabs((J.single ? hi : held(thr[0])) * unit) / step, -21);    // FP32 evaluation of the bytes
