@@ -1243,11 +1243,12 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                         }
                     }
                 }
-                // recorded while they are few enough to be used (D)
+                // recorded while they are few enough to be used (D); one lane reads the count for the
+                // warp, since other warps add to it meanwhile
                 const uint32_t fl = __ballot_sync(0xFFFFFFFFu, flip);
-                if (fl && record && *(volatile uint32_t*)n_flips <= (uint32_t)few) {
-                    int at = 0;
-                    if (lane == 0) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
+                if (fl && record) {
+                    int at = kFlips;
+                    if (lane == 0 && *(volatile uint32_t*)n_flips <= (uint32_t)few) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
                     at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(fl & ((1u << lane) - 1u));
                     if (flip && at < kFlips) flips[at] = (uint32_t)kl | ((uint32_t)f << 16);
                 }
