@@ -284,11 +284,11 @@ struct PlacementChoice {
 
 template <class FnOf>
 ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int dc_max, bool adapt, bool state,
-                              int limit, FnOf fn_of, PlacementChoice* out, int n_local = -1, bool many = false) {
+                              int limit, FnOf fn_of, PlacementChoice* out, int use = kLaunch, bool many = false) {
     using Key = std::vector<int64_t>;
     static std::mutex mu;
     static std::map<Key, PlacementChoice> cache;
-    const Key key = {dev, n, m, t_max, dv_max, dc_max, adapt, state, limit, n_local, many,
+    const Key key = {dev, n, m, t_max, dv_max, dc_max, adapt, state, limit, use, many,
                      (int64_t)(intptr_t)fn_of(true), (int64_t)(intptr_t)fn_of(false)};
     {
         std::lock_guard<std::mutex> g(mu);
@@ -300,6 +300,9 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
     }
     PlacementChoice best;
     int best_warps = 0;
+    // serving: with every chain entry's cutoff table if the kind fits so at all, else with one
+    for (const int u : {use, kTable + 1}) {
+    if (u != use && (use <= kTable || best.bps > 0 || dv_max > kNarrowDegree)) continue;
     for (const bool st : {true, false}) {
         if (st && !state) continue;
         const void* fn = fn_of(st);
@@ -310,8 +313,9 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
         if (best.bps > 0 && !(many && best.bps == 1)) break;
         const bool second = best.bps > 0;
         for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0, kTight}) {
-            if (tb == kTight && (best.bps > 0 || st || dv_max > kNarrowDegree)) continue;    // only where nothing else fits
-            const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, n_local);
+            // only where nothing else fits
+            if (tb == kTight && (best.bps > 0 || st || dv_max > kNarrowDegree || (use > kTable && u == use))) continue;
+            const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, -1, -1, u);
             if (L.total > limit) continue;
             for (const int block : {1024, 512, 256, kTightThreads}) {
                 if ((tb == kTight) != (block == kTightThreads)) continue;
@@ -331,6 +335,7 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
             }
         }
     }
+    }
     if (best.bps == 0) return fail(NGDBF_ERR_UNSUPPORTED, "code too large for the shared-memory decision words");
     std::lock_guard<std::mutex> g(mu);
     cache[key] = best;
@@ -349,13 +354,14 @@ ngdbf_status plan_smem(int dev, int n, int m, int t_max, int dv_max, int dc_max,
     PlacementChoice pc;
     ngdbf_status s = choose_placement(dev, n, m, t_max, dv_max, dc_max, adapt, state,
                                       smem_optin - (int)fa.sharedSizeBytes,
-                                      [&](bool st) { return st ? fn_st : fn_nost; }, &pc);
+                                      [&](bool st) { return st ? fn_st : fn_nost; }, &pc, kServe);
     if (s != NGDBF_OK) return s;
     out->st_smem = pc.st_smem;
     out->placement = pc.placement;
     out->block = pc.block;
     out->bps = pc.bps;
-    out->smem = pc.L.total;
+    // (one CTA per SM with fewer cutoff tables than chain entries: all the memory, for what more fit)
+    out->smem = pc.bps == 1 && pc.L.cuts > 0 && pc.L.cuts < kChain ? smem_optin - (int)fa.sharedSizeBytes : pc.L.total;
     return NGDBF_OK;
 }
 
@@ -373,7 +379,7 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     const bool many = !wide && !scarce_scratch && n_frames >= 2ll * sm_count * kSlots;
     ngdbf_status s = choose_placement(dev, C->n, C->m, P->t_max, C->dv_max, C->dc_max, adapt, state, smem_optin,
                                       [&](bool st) { return (const void*)pick_kernel(P->variant, P->precision, st, wide); },
-                                      &pc, -1, many);
+                                      &pc, kLaunch, many);
     if (s != NGDBF_OK) return s;
     KernelFn fn = pick_kernel(P->variant, P->precision, pc.st_smem, wide);
     const int best_block = pc.block, best_bps = pc.bps;

@@ -40,7 +40,7 @@ void host_gen_consts(uint64_t seed, GenConsts& G);
 size_t held_bytes(int precision);
 size_t slot_bytes(int precision, bool wide);
 ngdbf_status check_params(const ngdbf_params* P, float sigma);
-// Shared-memory plan of a kernel of the slot loop for the given maxima: per-slot state in
+// Shared-memory plan of a serving kernel for the given maxima: per-slot state in
 // shared memory when it fits (fn_st) else global (fn_nost), adjacency tables, block size.
 struct SmemPlan {
     bool st_smem;

@@ -92,7 +92,7 @@ constexpr int kTabChk = 1;              // N(i) table in shared memory
 constexpr int kTabSym = 2;              // M(k) table and degrees in shared memory
 // The longest codes (without their state in shared memory, and at most kTightThreads threads): the
 // warps' queues lie over the syndrome words, which phase C does not read, and flips are not
-// recorded (no D).  Every check has at most 64 symbols, so there are words enough.
+// recorded (no D).
 constexpr int kTight = 4;
 constexpr int kTightThreads = 128;
 
@@ -110,6 +110,10 @@ constexpr int kFlips = 256;
 // Bytes readable past a CTA's margin bytes (the last step of phase C reads whole warps of groups).
 constexpr int kMarginSlack = 32 * 32 * 4;
 constexpr int kQueue = 64;            // groups queued per warp for the exact form
+constexpr int kCutBytes = 256 * 4;    // one cutoff table
+// What a shared-memory layout is for (smem_layout): one job per launch, a job of a table, or a
+// serving CTA with cutoff tables for every chain entry (kTable + c: for c of them).
+constexpr int kLaunch = 0, kTable = 1, kServe = kTable + 8;
 // Single-bit: the least E_k is guessed kGuess noise scales above the last, the first kFirst above
 // the lowest tau followed, raised by kRaise at a time and to infinity after kSweeps sweeps.
 constexpr float kGuess = 1.5f, kFirst = 2.0f, kRaise = 2.0f;
@@ -198,6 +202,7 @@ struct Job {
 // slots hold (entries of jl, slot f holds a frame of jl[slot_e[f]]), the entry frames are
 // claimed from, and `next`, which finds another published job with the same chain_key.
 constexpr int kChain = 8;
+static_assert(kServe == kTable + kChain, "a cutoff table per chain entry");
 struct NoNext {
     __device__ bool operator()(unsigned long long, Job&) const { return false; }
 };
@@ -207,7 +212,15 @@ struct ChainCtx {
     int8_t* slot_e;             // [kSlots] shared memory
     int* cur_e;                 // shared memory
     Next next;
-    uint32_t* cut;              // [kChain][256] shared memory: cutoff table of each entry's job
+    int entries;                // entries in use: kChain, or the cutoff tables of the layout when fewer
+};
+
+// Static shared memory of the serving kernel.
+struct ServeShared {
+    Job jl[kChain];             // [0]: the request picked; the others: chained requests
+    unsigned long long fail[2];
+    int8_t slot_e[kSlots];
+    int cur_e, pick;
 };
 
 // Claims up to k consecutive frames of job A: returns true and the first frame id in *base
@@ -238,7 +251,7 @@ __device__ __forceinline__ bool claim_frames(const Job& A, unsigned k, unsigned 
 // Offsets in bytes of the shared-memory arrays (smem_layout).
 struct SmemLayout {
     int32_t off_frame, off_start, off_ctl, off_unsat, off_flips, off_best, off_tau, off_trace, off_icdf, off_cut, off_queue, off_xw, off_sw, off_cnt,
-        off_thr, off_st, off_chk, off_sym, total;
+        off_thr, off_st, off_chk, off_sym, cuts, total;
 };
 
 // Launch of one job: the job and its thresholds travel as kernel parameters.
@@ -305,9 +318,12 @@ __host__ __device__ inline int split_local_max(int n, int size) { return 32 * ((
 // and the zero sentinel word at index n.
 // `wide` (< 0: from dv_max) selects the count and syndrome formats, which follow the kernel's
 // WIDE template argument when a job table lays out a job of lower degree.
+// `use`: a launch of one job, a job of a table (no objective trace), or kServe cutoff tables of
+// a serving CTA, one per chain entry (no trace, and no second buffer of the single-bit minima,
+// which only CTAs of a cluster use).
 __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int dv_max, int dc_max,
                                                   bool need_thr, bool st_smem, int tables, int n_local = -1,
-                                                  int wide = -1) {
+                                                  int wide = -1, int use = kLaunch) {
     if (n_local < 0) n_local = n;   // symbols whose counts, state and M(k) rows this CTA holds
     const bool wd = wide < 0 ? dv_max > kNarrowDegree : wide != 0;
     SmemLayout L;
@@ -325,18 +341,21 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     const bool tight = (tables & kTight) != 0;
     // (wide: none of the lazy form's arrays)
     L.off_unsat = wd ? -1 : take(kSlots * 4, 16);   // number of unsatisfied checks of each slot
-    L.off_best = take(2 * kSlots * 8, 16); // single-bit variant: least (E key, k) per slot, two rounds
+    const int serve = use > kTable ? use - kTable : 0;      // cutoff tables asked for
+    L.off_best = take((serve ? 1 : 2) * kSlots * 8, 16);    // single-bit variant: least (E key, k) per slot, two rounds
     L.off_tau = wd ? -1 : take(kSlots * 4, 16);     // single-bit variant: guess of each slot's least E_k
-    L.off_trace = take(kSlots * 12, 16);   // objective trace: per slot C (int64), then U (int32)
+    L.off_trace = use == kLaunch ? take(kSlots * 12, 16) : -1;  // objective trace: per slot C (int64), then U (int32)
     L.off_icdf = take(256 * 16, 16);       // inverse normal CDF coefficients
-    L.off_cut = wd ? -1 : take(256 * 4, 16);        // cutoff of each margin byte
+    L.cuts = wd ? 0 : serve ? serve : 1;
+    L.off_cut = wd ? -1 : take(L.cuts * kCutBytes, 16);     // cutoff of each margin byte
     L.off_cnt = take(pad4(n_local) * cnt_bytes, 16);
     L.off_flips = wd || tight ? -1 : take(kFlips * 4, 16);   // flips of this iteration: local symbol | slot << 16
     // per warp: groups for the exact form (phase C's last steps may read up to 31 groups of counts
     // past the code's: they lie inside this array)
     L.off_queue = wd || tight ? -1 : take(32 * kQueue * 4, 16);
     L.off_xw = take(pad4(n + 1) * 4, 16);
-    L.off_sw = take((m + 1) * (wd ? 4 : 8), 16);
+    const int sw_bytes = (m + 1) * (wd ? 4 : 8), queues = kTightThreads / 32 * kQueue * 4;
+    L.off_sw = take(tight && sw_bytes < queues ? queues : sw_bytes, 16);
     if (tight) L.off_queue = L.off_sw;
     // all 512 values of the 9-bit u field: an idle slot's counter may pass T (its lookups are
     // don't-care but stay inside the table)
@@ -349,10 +368,10 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
 }
 
 // Layout L of a narrow or wide kernel with the offsets that do not depend on the code (all up to
-// the counts) as compile-time constants.
-template <bool WIDE>
+// the counts, or of a serving CTA to the cutoff tables) as compile-time constants.
+template <bool WIDE, int USE = kLaunch>
 __device__ __forceinline__ SmemLayout with_fixed_offsets(SmemLayout L) {
-    const SmemLayout F = smem_layout(4, 1, 0, 1, 1, false, false, 0, -1, WIDE ? 1 : 0);
+    const SmemLayout F = smem_layout(4, 1, 0, 1, 1, false, false, 0, -1, WIDE ? 1 : 0, USE);
     L.off_frame = F.off_frame;
     L.off_start = F.off_start;
     L.off_ctl = F.off_ctl;
@@ -362,25 +381,38 @@ __device__ __forceinline__ SmemLayout with_fixed_offsets(SmemLayout L) {
     L.off_trace = F.off_trace;
     L.off_icdf = F.off_icdf;
     L.off_cut = F.off_cut;
-    L.off_cnt = F.off_cnt;
+    if (USE <= kTable) L.off_cnt = F.off_cnt;
     return L;
 }
 
 // Layout of one job of a job table: arrays sized for the job's own code (n_local symbols per
 // CTA: its share when split over a cluster) in the launch's count and syndrome format, with
 // as many of the adjacency tables that `tables` allows as fit in `bytes` (both, then N(i)
-// alone, M(k) alone, none, then kTight without state); *tables_out receives the placement taken.  Host planning and the kernel
+// alone, M(k) alone, none, then kTight without state); *tables_out receives the placement taken.
+// A serving job (use > kTable) has a cutoff table for every chain entry if it fits so in any
+// of these ways but kTight; else for as many as fit, one at least.  Host planning and the kernel
 // evaluate it alike, so the launch's shared memory is the largest job's, not the layout of
 // the table's maxima.
 __host__ __device__ inline SmemLayout job_layout(int n, int m, int t_max, int dv_max, int dc_max, bool need_thr,
                                                  bool st_smem, bool wide, int tables, int n_local, int bytes,
-                                                 int* tables_out) {
+                                                 int* tables_out, int use = kTable) {
     const int opts[5] = {tables & (kTabChk | kTabSym), tables & kTabChk, tables & kTabSym, 0, kTight};
+    const bool serve = use > kTable;
     SmemLayout L{};
-    for (int i = 0; i < (wide || st_smem ? 4 : 5); ++i) {
-        L = smem_layout(n, m, t_max, dv_max, dc_max, need_thr, st_smem, opts[i], n_local, wide ? 1 : 0);
-        *tables_out = opts[i];
-        if (L.total <= bytes) break;
+    auto place = [&](int u, int n_opts) {
+        for (int i = 0; i < n_opts; ++i) {
+            L = smem_layout(n, m, t_max, dv_max, dc_max, need_thr, st_smem, opts[i], n_local, wide ? 1 : 0, u);
+            *tables_out = opts[i];
+            if (L.total <= bytes) return true;
+        }
+        return false;
+    };
+    // (with its state in shared memory only if every chain entry fits too)
+    if (!place(use, wide || st_smem || serve ? 4 : 5) && serve && !wide && !st_smem) place(kTable + 1, 5);
+    if (serve && L.cuts > 0 && L.total <= bytes) {       // the room left: more of the cutoff tables
+        const int more = (bytes - L.total) / kCutBytes, want = use - kTable - L.cuts;
+        L = smem_layout(n, m, t_max, dv_max, dc_max, need_thr, st_smem, *tables_out, n_local, 0,
+                        kTable + L.cuts + (more < want ? more : want));
     }
     return L;
 }
@@ -659,7 +691,7 @@ __device__ uint32_t fill_chained(ChainCtx<Next>& ch, unsigned long long key, uin
         // the current job has no frames left: another with the same key, into a free entry
         const uint32_t held = busy | fresh;
         int e2 = -1;
-        for (int e = 0; e < kChain && e2 < 0; ++e) {
+        for (int e = 0; e < ch.entries && e2 < 0; ++e) {
             if (e == *ch.cur_e) continue;
             bool used = false;
             for (uint32_t r = held; r; r &= r - 1) used |= ch.slot_e[__ffs(r) - 1] == e;
@@ -692,7 +724,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                                            const SmemLayout& L, int tables,
                                            typename Held<PREC>::T* ys, uint16_t* st_cta,
                                            Split S = Split{0, 1, 0, 0},
-                                           ChainCtx<Next> ch = ChainCtx<Next>{nullptr, nullptr, nullptr, Next{}, nullptr}) {
+                                           ChainCtx<Next> ch = ChainCtx<Next>{nullptr, nullptr, nullptr, Next{}, 0}) {
     static_assert(!(CL && CHAIN), "chained jobs are not split over clusters");
     constexpr bool kState = ADAPT || SMOOTH;
     // the job whose frame slot f holds (per-request fields: samples, sigma, frame offset,
@@ -729,7 +761,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     uint32_t* sw = reinterpret_cast<uint32_t*>(smem + L.off_sw);
     unsigned long long* best = reinterpret_cast<unsigned long long*>(smem + L.off_best);
     float4* icdf = reinterpret_cast<float4*>(smem + L.off_icdf);
-    uint32_t* cut = CHAIN ? ch.cut : reinterpret_cast<uint32_t*>(smem + L.off_cut);
+    uint32_t* cut = reinterpret_cast<uint32_t*>(smem + L.off_cut);
     float* tau = reinterpret_cast<float*>(smem + L.off_tau);
     const bool single = !ADAPT && A.single;
     // wide: every symbol evaluated, with its held sample in `ys`; else margin bytes there
@@ -830,7 +862,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     // threshold of the non-adaptive variants; chained jobs read it once here, since the first
     // job's memory is returned when that job completes
     const uint32_t th0_once = CHAIN ? __ldcg(thr_src) : 0u;
-    if (tid < 2 * kSlots) best[tid] = ~0ull;
+    if (tid < (CHAIN ? 1 : 2) * kSlots) best[tid] = ~0ull;
     if (split) {
         group_sync();        // every copy cleared before rank 0 writes the slot table
         if (tid == 0 && S.rank == 0) {

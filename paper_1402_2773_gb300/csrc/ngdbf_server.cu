@@ -135,14 +135,11 @@ template <bool ADAPT, bool SMOOTH, bool ST_SMEM, bool WIDE, int PREC>
 __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant__ ServeArgs A) {
     using HeldT = typename Held<PREC>::T;
     constexpr bool kState = ADAPT || SMOOTH;
-    __shared__ Job jl[kChain];      // jl[0]: the request picked; the others: chained requests
-    __shared__ int8_t slot_e[kSlots];
-    __shared__ int cur_e;
-    __shared__ unsigned long long fail[2];
-    __shared__ uint32_t cut[kChain * 256];      // cutoff tables of the entries
+    __shared__ ServeShared sh;
+    Job* const jl = sh.jl;
     Job& job = jl[0];
-    if (threadIdx.x == 0) fail[0] = fail[1] = ~0ull;
-    __shared__ int pick;
+    int& pick = sh.pick;
+    if (threadIdx.x == 0) sh.fail[0] = sh.fail[1] = ~0ull;
     HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, A.n_max);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_max) * kSlots : nullptr;
     const volatile ServeRing* R = A.ring;
@@ -197,23 +194,25 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
         slept = 0;
         nap = 500;
         int tables = 0;
-        const ChainCtx<RingNext> ch{jl, slot_e, &cur_e, RingNext{R, fail}, cut};
+        ChainCtx<RingNext> ch{jl, sh.slot_e, &sh.cur_e, RingNext{R, sh.fail}, kChain};
         bool done = false;
         if constexpr (kState && !ST_SMEM && !WIDE) {
             const SmemLayout Ls = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT, true, WIDE,
-                                             A.placement, job.n, A.smem_bytes, &tables);
+                                             A.placement, job.n, A.smem_bytes, &tables, kServe);
             if (Ls.total <= A.smem_bytes) {
+                ch.entries = Ls.cuts;
                 decode_job<ADAPT, SMOOTH, true, WIDE, PREC, false, true, RingNext>(
-                    job, job.thr, A.G, Ls, tables, ys, nullptr, Split{0, 1, 0, 0}, ch);
+                    job, job.thr, A.G, with_fixed_offsets<WIDE, kServe>(Ls), tables, ys, nullptr, Split{0, 1, 0, 0}, ch);
                 done = true;
             }
         }
         if (!done) {
             // (a code no larger than the kind's maxima always fits without its state)
             const SmemLayout L = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT,
-                                            ST_SMEM && kState, WIDE, A.placement, job.n, A.smem_bytes, &tables);
+                                            ST_SMEM && kState, WIDE, A.placement, job.n, A.smem_bytes, &tables, kServe);
+            if constexpr (!WIDE) ch.entries = L.cuts;
             decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC, false, true, RingNext>(
-                job, job.thr, A.G, L, tables, ys, st, Split{0, 1, 0, 0}, ch);
+                job, job.thr, A.G, with_fixed_offsets<WIDE, kServe>(L), tables, ys, st, Split{0, 1, 0, 0}, ch);
         }
         __syncthreads();
     }
