@@ -497,8 +497,9 @@ ngdbf_status launch_kernel(ngdbf_server* S) {
 }
 
 // The kind a kernel needs for the first request to admit: the largest layout of its variant and
-// precision seen so far (so that the kernel rarely has to drain for a larger code).
-Kind kind_for(ngdbf_server* S, const Request* first) {
+// precision seen so far (so that the kernel rarely has to drain for a larger code), or `alone`, its
+// own, forgetting those (their maxima together do not fit).
+Kind kind_for(ngdbf_server* S, const Request* first, bool alone = false) {
     const ngdbf_job& f = first->job;
     Kind* K = nullptr;
     for (Kind& k : S->seen)
@@ -520,7 +521,9 @@ Kind kind_for(ngdbf_server* S, const Request* first) {
         K->dv = std::max(K->dv, q.code->dv_max);
         K->dc = std::max(K->dc, q.code->dc_max);
     };
+    if (alone) K->n = K->m = K->t_max = K->dv = K->dc = 0;
     grow(f);
+    if (alone) return *K;
     for (Request* r : S->pending) grow(r->job);
     return *K;
 }
@@ -611,7 +614,13 @@ void scheduler(ngdbf_server* S) {
             if (!on_device) {
                 K = kind_for(S, r);
                 ServePlan P;
-                if (plan_serve(S, K, &P) != NGDBF_OK) {
+                ngdbf_status s = plan_serve(S, K, &P);
+                if (s != NGDBF_OK) {
+                    // maxima over several codes can exceed what each of them needs: a kind of its own
+                    K = kind_for(S, r, true);
+                    s = plan_serve(S, K, &P);
+                }
+                if (s != NGDBF_OK) {
                     S->pending.pop_front();
                     finish(S, r, NGDBF_ERR_UNSUPPORTED);
                     progressed = true;

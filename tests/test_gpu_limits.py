@@ -77,3 +77,24 @@ def test_table_takes_the_longest_codes(O, n, m):
         batch.close()
         for c in codes:
             c.close()
+
+
+def test_codes_whose_maxima_do_not_fit_together(O):
+    """Two codes that fit alone, one of many symbols and one of many checks: a kernel for both would
+    need more shared memory than there is, so the server serves them in turn."""
+    A = long_code(9300, 930)
+    H = np.zeros((5590, 5600), np.uint8)
+    H[np.arange(5600) % 5590, np.arange(5600)] = 1
+    H[10:20, 0] = 1
+    B = wl.code_from_dense(H)
+    reqs, want = [], []
+    for j, code in enumerate([A, B, A, B, B, A]):
+        gp, op = params_pair(variant=3, lam=0.95, t_max=6, smooth_window=3, w=0.4, theta=-0.5)
+        y, _, _ = wl.frames(code, 4, None, seed=50 + j, sigma=0.7)
+        reqs.append((code, y, 0.7, gp, 100 * j))
+        want.append(O.decode_f32(code, y, 0.7, op, seed=4, frame_offset=100 * j, threads=THREADS))
+    outs, status = serve(reqs, seed=4)
+    assert status == [0] * len(reqs)
+    for got, ref in zip(outs, want):
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b)
