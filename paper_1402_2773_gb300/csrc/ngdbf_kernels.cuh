@@ -896,7 +896,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             // (four samples in flight per thread)
             const uint32_t fresh = ctl[3];
             if (!dense && single && tid < kSlots && ((fresh >> tid) & 1u)) tau[tid] = A.pf_low + kFirst * job_of(tid).scale;
-            if constexpr (CHAIN) {
+            if constexpr (CHAIN && !WIDE) {
                 for (uint32_t r = ctl[4]; r; r &= r - 1) {
                     const int e = __ffs(r) - 1;
                     for (int i = tid; i < 256; i += blockDim.x) cut[256 * e + i] = margin_cutoff(i, ch.jl[e]);
