@@ -226,8 +226,15 @@ void host_gen_consts(uint64_t seed, GenConsts& G) {
     std::memcpy(G.icdf, table.words(), sizeof(G.icdf));
 }
 
+// Fewest frames for which a small batch takes one more CTA.  In the lazy form a CTA's time per
+// iteration grows with its live slots, so a small batch takes every CTA that can be resident as long
+// as each gets a frame.  The dense form of wide codes has a lane per slot, live or not: packed 32
+// to a CTA it takes the same time on a 32nd of the SMs (degree 20, n = 512: 500 frames 0.73 ms
+// packed, 1.15 spread; 64 streams of 96 frames 47 ms packed, 235 spread).
+int spread_least(bool wide) { return wide ? kSlots : 1; }
+
 struct LaunchPlan {
-    int block, grid, blocks_per_sm, smem;
+    int block, grid, blocks_per_sm, smem, slots_least;
     bool st_smem;
     int placement;              // adjacency tables in shared memory: kTabChk | kTabSym
 };
@@ -388,9 +395,8 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     const int placement = pc.placement;
     plan->block = best_block;
     plan->blocks_per_sm = best_bps;
-    // every CTA that can be resident, as long as each gets a frame: a CTA's time per iteration
-    // grows with its live slots, so a small batch is spread over the SMs, not packed 32 to a CTA
-    plan->grid = (int)std::min<int64_t>((int64_t)sm_count * best_bps, n_frames);
+    plan->slots_least = spread_least(wide);
+    plan->grid = (int)std::min<int64_t>((int64_t)sm_count * best_bps, (n_frames + plan->slots_least - 1) / plan->slots_least);
     plan->smem = L.total;
     plan->st_smem = st_smem;
     plan->placement = placement;
@@ -523,10 +529,10 @@ void fill_job(const ngdbf_code* C, const ngdbf_params* P, const float* y, int64_
     fill_margins(C, P, thr, &J);
 }
 
-// Frames a CTA takes first when n_frames are decoded by n_ctas CTAs.
-int first_slots(int64_t n_frames, int64_t n_ctas) {
+// Frames a CTA takes first when n_frames are decoded by n_ctas CTAs, `least` at least (spread_least).
+int first_slots(int64_t n_frames, int64_t n_ctas, int least) {
     const int64_t per = (n_frames + n_ctas - 1) / std::max<int64_t>(n_ctas, 1);
-    return (int)std::min<int64_t>(std::max<int64_t>(per, 1), kSlots);
+    return (int)std::min<int64_t>(std::max<int64_t>(per, least), kSlots);
 }
 
 // Kernel arguments of one decode: scratch at `base` (work counter, then the
@@ -540,7 +546,7 @@ void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& pla
     fill_job(C, P, y, n_frames, sigma, frame_offset, bits, iters, pass,
              reinterpret_cast<unsigned long long*>(base), &A.J, A.thr);
     A.J.thr = nullptr;                 // thresholds travel inline in the launch
-    A.J.slots = first_slots(n_frames, grid);
+    A.J.slots = first_slots(n_frames, grid, plan.slots_least);
     A.placement = plan.placement;
     A.L = smem_layout(C->n, C->m, P->t_max, C->dv_max, C->dc_max, (P->variant & NGDBF_ADAPT) != 0,
                       plan.st_smem && (P->variant & 3) != 0, plan.placement);
@@ -636,6 +642,7 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
         cudaGetLastError();
         s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count, true);
         if (s != NGDBF_OK) return s;
+        plan.slots_least = kSlots;
         plan.grid = (int)std::min<int64_t>(plan.grid, (n_frames + kSlots - 1) / kSlots);
         e = take_scratch();
     }
@@ -1052,6 +1059,7 @@ extern "C" ngdbf_status ngdbf_decode_noalloc(const ngdbf_code_t* C, const float*
 
 struct ngdbf_batch {
     int device = 0, n_jobs = 0, sm_count = 0;
+    bool wide = false;                  // bit-sliced counts (TablePlan::wide)
     void* fn = nullptr;                 // job-table kernel
     int grid = 0, block = 0, smem = 0, state_in_smem = 0, tables_in_smem = 0, cluster = 1;
     MultiArgs args;
@@ -1344,7 +1352,7 @@ cudaError_t batch_enqueue(ngdbf_batch* B, cudaStream_t stream) {
 
 // Puts candidate `k` in use: kernel, launch shape, shared-memory plan, the first job of every CTA
 // (of every cluster: a split job can use one cluster per frame, a job decoded CTA by CTA one
-// cluster per C frames) and the frames a CTA takes first of each job.
+// cluster per C frames; 32 times as many for wide codes) and the frames a CTA takes first of each job.
 ngdbf_status batch_set_shape(ngdbf_batch* B, int k) {
     const TableShape& sh = B->shapes[k];
     const int C = sh.cluster;
@@ -1364,7 +1372,7 @@ ngdbf_status batch_set_shape(ngdbf_batch* B, int k) {
     std::vector<int64_t> cap(B->n_jobs);
     int64_t clusters = 0;
     for (int j = 0; j < B->n_jobs; ++j) {
-        const int64_t per = B->n_of_job[j] >= sh.split_min_n ? 1 : C;
+        const int64_t per = (B->n_of_job[j] >= sh.split_min_n ? 1 : C) * spread_least(B->wide);
         cap[j] = (B->frames[j] + per - 1) / per;
         clusters += cap[j];
     }
@@ -1374,7 +1382,7 @@ ngdbf_status batch_set_shape(ngdbf_batch* B, int k) {
     std::vector<int32_t> slots(B->n_jobs, 1);
     for (int j = 0; j < B->n_jobs; ++j) {
         const int64_t cls = std::max<int64_t>(1, std::count(first.begin(), first.end(), j));
-        slots[j] = first_slots(B->frames[j], cls * (B->n_of_job[j] >= sh.split_min_n ? 1 : C));
+        slots[j] = first_slots(B->frames[j], cls * (B->n_of_job[j] >= sh.split_min_n ? 1 : C), spread_least(B->wide));
     }
     cudaError_t e = cudaMemcpy(B->d_first, first.data(), first.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(B->d_slots, slots.data(), slots.size() * 4, cudaMemcpyHostToDevice);
@@ -1439,6 +1447,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     B->device = dev;
     B->n_jobs = n_jobs;
     B->sm_count = T.sm_count;
+    B->wide = T.wide;
     ngdbf_status ss = table_shapes(T, jobs, n_jobs, dev, &B->shapes);
     if (ss != NGDBF_OK) { batch_free(B); return ss; }
     // scratch for the largest candidate: per CTA the samples (and state) of its symbols

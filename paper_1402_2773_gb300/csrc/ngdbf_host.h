@@ -90,8 +90,10 @@ void staging_release(Staging* s);
 // the device copies out of it; returns when the last piece is queued.
 cudaError_t staged_h2d(Staging* s, void* dst, const void* src, size_t bytes, cudaStream_t st);
 
-// Frames a CTA takes first when n_frames are decoded by n_ctas CTAs (Job::slots).
-int first_slots(int64_t n_frames, int64_t n_ctas);
+// Frames a CTA takes first when n_frames are decoded by n_ctas CTAs (Job::slots), at least `least`;
+// the fewest frames for which a small batch takes one more CTA.
+int first_slots(int64_t n_frames, int64_t n_ctas, int least);
+int spread_least(bool wide);
 
 // First job of every CTA, in proportion to the estimated work of each job.
 std::vector<int32_t> assign_ctas(const std::vector<int64_t>& frames, const std::vector<int64_t>& weight, int grid);

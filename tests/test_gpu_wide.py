@@ -1,13 +1,14 @@
 """Symbol degrees above 15 (bit-sliced counts, every E_k formed) through every kernel vs the
 reference decoder, bit for bit: single launches with full slots, job tables that hold narrow and
-wide codes in every launch shape (clusters too), and the server.
+wide codes in every launch shape (clusters too), and the server.  A small batch of such a code
+is packed 32 frames to a CTA, whose time does not depend on its live slots.
 """
 import numpy as np
 import pytest
 
 from paper_1402_2773_gb300 import ngdbf, workload as wl
 from test_gpu_limits import serve
-from test_gpu_parity import O, _gpu, params_pair, THREADS  # noqa: F401
+from test_gpu_parity import O, _gpu, gpu_decode, params_pair, THREADS  # noqa: F401
 from test_gpu_slots import assert_slots
 from test_z_lazy import PREC, code_with_degree
 
@@ -24,6 +25,35 @@ def job(O, code, F, variant, prec, j):
     gp, op = params_pair(variant=variant, **KW, **prec)
     y, _, _ = wl.frames(code, F, None, seed=70 + j, sigma=0.6)
     return (code, y, gp, 1000 * j, O.decode_f32(code, y, 0.6, op, seed=9, frame_offset=1000 * j, threads=THREADS))
+
+
+@pytest.mark.parametrize("F", [1, 32, 33, 96, 500])
+def test_small_batches_are_packed(O, F):
+    gp, op = params_pair(variant=3, **KW)
+    y, _, _ = wl.frames(W20, F, None, seed=7, sigma=0.6)
+    got = gpu_decode(W20, y, 0.6, gp, 3)
+    assert ngdbf.ngdbf_last_launch()["grid"] == (F + 31) // 32
+    for a, b in zip(got, O.decode_f32(W20, y, 0.6, op, seed=3, threads=THREADS)):
+        assert np.array_equal(a, b)
+
+
+def test_small_jobs_of_a_table_are_packed(O):
+    """The first shape (no cluster): a CTA per 32 frames of each job."""
+    made = [job(O, code, F, 3, {}, j) for j, (code, F) in enumerate([(W20, 33), (W16, 64), (NARROW, 70)])]
+    codes = [ngdbf.DeviceCode.from_code(q[0]) for q in made]
+    batch = ngdbf.Batch([(dc, torch.from_numpy(q[1]).cuda(), 0.6, q[2], q[3]) for dc, q in zip(codes, made)], seed=9)
+    try:
+        batch.use_shape(0)
+        got = batch.launch()
+        torch.cuda.synchronize()
+        assert ngdbf.ngdbf_last_launch()["grid"] == 2 + 2 + 3
+        for g, q in zip(got, made):
+            for a, b in zip(g, q[4]):
+                assert np.array_equal(a.cpu().numpy(), b)
+    finally:
+        batch.close()
+        for dc in codes:
+            dc.close()
 
 
 @pytest.mark.parametrize("prec", PREC, ids=["fp32", "fp16", "fix3", "fixacc8"])
