@@ -151,9 +151,10 @@ ngdbf_status ngdbf_code_info(const ngdbf_code_t* code, int32_t* n, int32_t* m,
  *   stream       cudaStream_t to run on (NULL = legacy default stream)
  * Asynchronous: returns after enqueueing; outputs are valid once the stream
  * reaches this point; y must stay unchanged until then (it is read while
- * frames are decoded).  Temporary device memory (per-slot margins, for large
- * batches and long codes the per-slot state, and a work counter: 32 to 96 * n
- * bytes per resident CTA) is taken from a library-owned stream-ordered pool
+ * frames are decoded).  Temporary device memory (per-slot samples or margins:
+ * 128 n bytes per resident CTA in FP32, 64 n in FP16, 32 n in fixed point; 64 n
+ * more where the per-slot state is in global memory, for large batches and long
+ * codes; and 5 KB) is taken from a library-owned stream-ordered pool
  * and returned on the same stream.  All pointers must be device memory of the current device.
  * The decision, syndrome and count words of one CTA's 32 frames must fit the
  * device's shared memory per block (about 20 n + 8 m + 7 KB bytes for symbol

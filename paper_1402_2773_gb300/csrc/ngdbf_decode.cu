@@ -73,7 +73,7 @@ template <bool ADAPT, bool SMOOTH, bool ST_SMEM, bool WIDE, int PREC>
 __global__ void __launch_bounds__(1024) ngdbf_persistent_kernel(const __grid_constant__ DecodeArgs A) {
     using HeldT = typename Held<PREC>::T;
     const Job& J = A.J;
-    HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, J.n);
+    HeldT* ys = slot_scratch<PREC>(A.yslots, blockIdx.x, J.n);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(J.n) * kSlots : nullptr;
     decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, with_fixed_offsets<WIDE>(A.L), A.placement, ys, st);
 }
@@ -266,10 +266,7 @@ KernelFn pick_kernel(int variant, int precision, bool st_smem, bool wide) {
     }
 }
 
-// Bytes of slot scratch per (symbol, slot): the margin byte, or the held sample of wide codes.
-size_t slot_bytes(int precision, bool wide) { return wide ? held_bytes(precision) : 1; }
-
-// Bytes of one held sample.
+// Bytes of one held sample: the slot scratch per (symbol, slot).
 size_t held_bytes(int precision) {
     return precision == NGDBF_FP16 ? 2 : ((precision == NGDBF_FIX || precision == NGDBF_FIXACC) ? 1 : 4);
 }
@@ -632,7 +629,7 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     void* ws = nullptr;
     auto take_scratch = [&]() {
         const size_t slot_elems = (size_t)plan.grid * pad4(C->n) * kSlots;
-        bytes_y = align256(slot_elems * slot_bytes(P->precision, C->dv_max > kNarrowDegree));
+        bytes_y = align256(slot_elems * held_bytes(P->precision));
         bytes_st = (state && !plan.st_smem) ? align256(slot_elems * 2) : 0;
         return cudaMallocFromPoolAsync(&ws, 256 + bytes_y + bytes_st + kMarginSlack, pool, stream);
     };
@@ -732,7 +729,7 @@ ngdbf_status ngdbf_code_create(int32_t n, int32_t m, const int32_t* row_ptr, con
     // M(k) by groups of four symbols [j][k/4][k%4], padded with the zero-word sentinel m, so that
     // one 8-byte load gives the j-th check of the four symbols of a group
     std::vector<uint16_t> sym((size_t)pad4(n) * dv_max, (uint16_t)m);
-    std::vector<uint8_t> deg(n);
+    std::vector<uint8_t> deg(pad4(n), 0);     // (read in words of four)
     std::vector<int32_t> fill(n, 0);
     for (int i = 0; i < m; ++i)
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
@@ -1454,7 +1451,7 @@ extern "C" ngdbf_status ngdbf_batch_create(const ngdbf_job* jobs, int32_t n_jobs
     size_t grid_max = 0, bytes_y = 0, bytes_st = 0;
     for (const TableShape& sh : B->shapes) {
         grid_max = std::max(grid_max, (size_t)sh.grid_max);
-        bytes_y = std::max(bytes_y, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * slot_bytes(T.precision, T.wide));
+        bytes_y = std::max(bytes_y, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * held_bytes(T.precision));
         if (sh.state_global) bytes_st = std::max(bytes_st, (size_t)sh.grid_max * pad4(sh.n_local) * kSlots * 2);
     }
     const size_t off_jobs = 0, off_thr = align256(sizeof(Job) * n_jobs), off_q = off_thr + align256(T.thr_words * 4);

@@ -48,7 +48,8 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
 // g and are formed once, which leaves 18 of the 20 wide multiplies per call.
 struct PhiloxLane {
     uint32_t fhi, lo1, h0, l0;
-    __device__ __forceinline__ PhiloxLane(uint64_t frame, uint32_t t, const GenConsts& G) {
+    template <class Keys>       // (rk0, rk1 as in GenConsts)
+    __device__ __forceinline__ PhiloxLane(uint64_t frame, uint32_t t, const Keys& G) {
         fhi = (uint32_t)(frame >> 32);
         const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint32_t)frame;
         const uint64_t q0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ t ^ G.rk0[0]);
@@ -56,7 +57,8 @@ struct PhiloxLane {
         h0 = (uint32_t)(q0 >> 32) ^ G.rk1[1];
         l0 = (uint32_t)q0;
     }
-    __device__ __forceinline__ void group(uint32_t g, const GenConsts& G, uint32_t out[4]) const {
+    template <class Keys>
+    __device__ __forceinline__ void group(uint32_t g, const Keys& G, uint32_t out[4]) const {
         const uint64_t p0 = (uint64_t)0xD2511F53u * g;
         const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(p0 >> 32) ^ fhi ^ G.rk1[0]);
         uint32_t c0 = (uint32_t)(p1 >> 32) ^ lo1, c1 = (uint32_t)p1, c2 = h0 ^ (uint32_t)p0, c3 = l0;

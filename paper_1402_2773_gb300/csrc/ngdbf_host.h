@@ -36,9 +36,8 @@ size_t align256(size_t v);
 ngdbf_status get_pool(int dev, cudaMemPool_t* out);
 // Philox round keys and series coefficients of the perturbation generator.
 void host_gen_consts(uint64_t seed, GenConsts& G);
-// Bytes of one held sample of a precision; of slot scratch per (symbol, slot).
+// Bytes of one held sample of a precision: the slot scratch per (symbol, slot).
 size_t held_bytes(int precision);
-size_t slot_bytes(int precision, bool wide);
 ngdbf_status check_params(const ngdbf_params* P, float sigma);
 // Shared-memory plan of a serving kernel for the given maxima: per-slot state in
 // shared memory when it fits (fn_st) else global (fn_nost), adjacency tables, block size.

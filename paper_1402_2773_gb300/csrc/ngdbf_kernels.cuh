@@ -19,7 +19,8 @@
 //      that no flip can exceed (see "Lazy evaluation"); the few outputs at or below
 //      it are queued and only for those E_k = x_k y_k + w S_k + q_k is formed and
 //      compared with theta lambda^{u_k} (Step 3a: with the slot's least so far).  Symbol
-//      degrees above 15 form E_k for every symbol, with lane = slot.
+//      degrees above 15 form E_k for every symbol, with lane = slot, and so do iterations in
+//      which about a sixth of the outputs or more would be evaluated (full_rounds).
 // When an iteration flipped few decisions (at most kFlips, a code not split over a cluster),
 // A and A' are replaced by
 //   D. per flip, its d_v checks toggled for the slot, the slot's number of unsatisfied checks
@@ -28,8 +29,8 @@
 // converged frame frees its slot at once, and the CTA only stops when the
 // queue is empty and its last slot finished.
 //
-// Per-(symbol, slot) state: one byte of quantized margin (global scratch, L2-resident; the
-// dense forms hold the sample itself there), and a 16-bit word holding the flips of the symbol
+// Per-(symbol, slot) state: one byte of quantized margin (global scratch, L2-resident; while every
+// E_k is formed the held sample is there instead), and a 16-bit word holding the flips of the symbol
 // so far (bits 0-8; u_k = t - flips) and the number of -1 decisions the smoothing window will
 // have seen at T if the symbol flips no more (bits 9-15), in shared memory when it fits, else
 // in global scratch.  Both change only when a symbol flips.  Both are laid out by groups of
@@ -111,6 +112,11 @@ constexpr int kFlips = 256;
 constexpr int kMarginSlack = 32 * 32 * 4;
 constexpr int kQueue = 64;            // groups queued per warp for the exact form
 constexpr int kCutBytes = 256 * 4;    // one cutoff table
+// Outputs evaluated per group of 32 slots (of 128) in one iteration, looked at in every fourth, above which
+// every E_k is formed from the next one on (full_rounds).  The exact form takes about 125 cycles of an SM
+// per 32 outputs, forming every E_k about 75 cycles more than the sweep per group, so the two meet near a
+// sixth of the outputs: between 2.0 and 2.5 dB for the (3,6) code of 1008 symbols (12 and 20 measured alike).
+constexpr int kFullMarks = 16, kFullEvery = 3;
 // What a shared-memory layout is for (smem_layout): one job per launch, a job of a table, or a
 // serving CTA with cutoff tables for every chain entry (kTable + c: for c of them).
 constexpr int kLaunch = 0, kTable = 1, kServe = kTable + 8;
@@ -130,13 +136,11 @@ template <> struct Held<kFP16> { using T = __half; };
 template <> struct Held<kFIX> { using T = int8_t; };      // signed level code b, value 2b + 1
 template <> struct Held<kFIXACC> { using T = int8_t; };   // the same Eq. 8 level code
 
-// Bytes of slot scratch per (symbol, slot): the margin byte, or with bit-sliced counts (wide) the
-// held sample; and the scratch of CTA `cta` of a launch whose CTAs hold n symbols each.
-template <int PREC, bool WIDE>
+// Slot scratch of CTA `cta` of a launch whose CTAs hold n symbols each: room for a held sample per
+// (symbol, slot), whose first part the margin bytes take.
+template <int PREC>
 __device__ __forceinline__ typename Held<PREC>::T* slot_scratch(void* base, int cta, int n) {
-    using T = typename Held<PREC>::T;
-    const size_t at = (size_t)cta * pad4(n) * kSlots;
-    return WIDE ? static_cast<T*>(base) + at : reinterpret_cast<T*>(static_cast<uint8_t*>(base) + at);
+    return static_cast<typename Held<PREC>::T*>(base) + (size_t)cta * pad4(n) * kSlots;
 }
 
 // One decode job: a code, a batch of frames and the parameters of the method.
@@ -258,7 +262,7 @@ struct SmemLayout {
 struct DecodeArgs {
     Job J;
     int32_t placement;          // adjacency tables copied into shared memory: kTabChk | kTabSym
-    void* yslots;               // [grid][pad4(n)/4][32][4] margin bytes (wide: held samples of 4, 2 or 1 bytes)
+    void* yslots;               // [grid][pad4(n)/4][32][4] margin bytes, or held samples of 4, 2 or 1 bytes
     uint16_t* st_global;        // [grid][pad4(n)/4][32][4] when the state is not in shared memory
     SmemLayout L;
     GenConsts G;
@@ -362,7 +366,7 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int m, int t_max, int d
     L.off_thr = need_thr ? take((kUMask + 1) * 4, 16) : -1;
     L.off_st = st_smem ? take(pad4(n_local) * kSlots * 2, 16) : -1;
     L.off_chk = (tables & kTabChk) ? take(chk_entries(m, dc_max) * 2, 16) : -1;
-    L.off_sym = (tables & kTabSym) ? take(pad4(n_local) * dv_max * 2 + n_local, 16) : -1;
+    L.off_sym = (tables & kTabSym) ? take(pad4(n_local) * dv_max * 2 + pad4(n_local), 16) : -1;
     L.total = (o + 15) / 16 * 16;
     return L;
 }
@@ -512,18 +516,28 @@ __device__ __forceinline__ float read_sample(const Job& A, long long frame, int 
 template <int PREC> struct Metric { using T = int32_t; };
 template <> struct Metric<kFP32> { using T = float; };
 template <> struct Metric<kFP16> { using T = float; };
-template <int PREC>
-__device__ __forceinline__ typename Metric<PREC>::T metric(typename Held<PREC>::T h, uint32_t xsign, int S, float q,
-                                                           const Job& A) {
+// (S is an integer or the float of the same value.)
+__device__ __forceinline__ float as_float(int S) { return __int2float_rn(S); }
+__device__ __forceinline__ float as_float(float S) { return S; }
+// What metric() takes from a job.
+struct MetricConsts {
+    float w, fix_R;
+    int32_t fix_kmax, fix_W;
+    float acc_R;
+    int32_t acc_W;
+};
+template <int PREC, class Sum, class Consts>
+__device__ __forceinline__ typename Metric<PREC>::T metric(typename Held<PREC>::T h, uint32_t xsign, Sum S, float q,
+                                                           const Consts& A) {
     if constexpr (PREC == kFP32) {
         const float xy = __uint_as_float(__float_as_uint(h) ^ xsign);
-        return __fadd_rn(__fadd_rn(xy, __fmul_rn(A.w, __int2float_rn(S))), q);
+        return __fadd_rn(__fadd_rn(xy, __fmul_rn(A.w, as_float(S))), q);
     } else if constexpr (PREC == kFP16) {
         // fl(w S_k) is the exact product of a binary16 w and a small integer; the additions are
         // binary16 additions (a correctly rounded FP32 addition of binary16 operands rounded
         // once more to binary16 gives the same value)
         const __half xy = __ushort_as_half(__half_as_ushort(h) ^ (uint16_t)(xsign >> 16));
-        const float ws = __fmul_rn(A.w, __int2float_rn(S));
+        const float ws = __fmul_rn(A.w, as_float(S));
         return __half2float(__hadd(__hadd(xy, __float2half_rn(ws)), __float2half_rn(q)));
     } else if constexpr (PREC == kFIX) {
         // Eq. 9 in units of Delta/2, exact integers
@@ -652,6 +666,241 @@ __device__ __forceinline__ void load_held4(const int8_t* p, int8_t v[4]) {
     const uint32_t a = *reinterpret_cast<const uint32_t*>(p);
     v[0] = (int8_t)(a & 0xFFu); v[1] = (int8_t)((a >> 8) & 0xFFu);
     v[2] = (int8_t)((a >> 16) & 0xFFu); v[3] = (int8_t)(a >> 24);
+}
+
+// State word of a symbol after a flip at the slot's iteration t: the flip count, and the window
+// count, which takes the new decision for x(t + 1) .. x(T).
+template <bool ADAPT, bool SMOOTH>
+__device__ __forceinline__ uint32_t flipped_state(uint32_t s0, bool was_neg, int t, int t_max, int t_smooth) {
+    uint32_t s1 = s0 + (ADAPT ? 1u : 0u);
+    if constexpr (SMOOTH) {
+        const uint32_t rem = (uint32_t)(t_max - max(t + 1, t_smooth) + 1) << kCShift;
+        s1 = was_neg ? s1 - rem : s1 + rem;
+    }
+    return s1;
+}
+
+// Phase A' (narrow): two threads per group, each for 16 slots: the four symbols' check words added in
+// 2-bit lanes three at a time, widened to nibbles (even and odd slots), and the bytes of the four
+// symbols gathered into the words that phase C reads.  unit(i, e, d): the (e + d)-th checks of the
+// group's symbols, for task i.
+template <class Unit>
+__device__ __forceinline__ void count_groups(uint4* cnt, const uint32_t* sw, int groups, int dv_max, Unit unit) {
+    for (int i = threadIdx.x; i < 2 * groups; i += blockDim.x) {
+        const int gl = i >> 1, h = i & 1;
+        uint32_t ev[4] = {0u, 0u, 0u, 0u}, od[4] = {0u, 0u, 0u, 0u};
+        for (int e = 0; e < dv_max; e += 3) {
+            uint32_t a[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                if (e + d >= dv_max) break;
+                const uint2 c = unit(i, e, d);
+                a[0] += sw[2 * (c.x & 0xFFFFu) + h];
+                a[1] += sw[2 * (c.x >> 16) + h];
+                a[2] += sw[2 * (c.y & 0xFFFFu) + h];
+                a[3] += sw[2 * (c.y >> 16) + h];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                ev[j] += a[j] & 0x33333333u;
+                od[j] += (a[j] >> 2) & 0x33333333u;
+            }
+        }
+        auto bytes = [](const uint32_t w[4]) {      // word b: byte b of w[0..3]
+            const uint32_t t0 = __byte_perm(w[0], w[1], 0x5140), t1 = __byte_perm(w[0], w[1], 0x7362);
+            const uint32_t u0 = __byte_perm(w[2], w[3], 0x5140), u1 = __byte_perm(w[2], w[3], 0x7362);
+            return make_uint4(__byte_perm(t0, u0, 0x5410), __byte_perm(t0, u0, 0x7632),
+                              __byte_perm(t1, u1, 0x5410), __byte_perm(t1, u1, 0x7632));
+        };
+        cnt[4 * gl + 2 * h] = bytes(ev);
+        cnt[4 * gl + 2 * h + 1] = bytes(od);
+    }
+}
+
+// Philox round keys as PhiloxLane takes them.
+struct PhiloxKeys {
+    uint32_t rk0[10], rk1[10];
+};
+
+// Iterations with every E_k formed (narrow codes not split over a cluster, Step 3b, no trace), lane =
+// slot, for a CTA of more than 16 live slots of whose outputs so many are at or below their cutoffs
+// that the exact form of those one by one costs more.  Takes over after phase C of iteration `round`,
+// in which tally[0] outputs were evaluated; runs phases A, A' and C until a slot finishes or the flips
+// say that few outputs would be evaluated, and returns the iteration whose phase A is next.  The slots'
+// held samples take the place of their margins in the scratch, and at the end the margins theirs.  A
+// function of its own, so that the lazy loop's registers and code are what they are without it.
+// 20000 frames, T = 300, all evaluated one by one before this, the former dense form in brackets: (3,6)
+// code of 1008 symbols at 0 dB 29.3 -> 18.2 ms (17.2), 1.0 dB 26.4 -> 17.5 (17.2), 2.0 dB 20.0 -> 15.9
+// (16.4), 2.5 dB 9.4 (11.9); (6,32) code of 2048 at 2.0 dB 37.5 -> 32.7 (36.8), 3.0 dB 32.1 -> 30.4 (36.8).
+template <bool ADAPT, bool SMOOTH, bool ST_SMEM, int PREC, bool CHAIN>
+__device__ __noinline__ int full_rounds(const Job& A, const Job* jl, const int8_t* slot_e, int off_icdf, int off_cnt,
+                                        int off_xw, int off_sw, int off_thr, int off_st, const uint16_t* chk_cols, const uint16_t* sym_chks, const uint8_t* sym_deg,
+                                        int sym_groups, typename Held<PREC>::T* ys, uint16_t* st_cta, uint32_t th0, int round) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr bool kState = ADAPT || SMOOTH;
+    // (the offsets ahead of the single-bit minima are the same in every narrow layout)
+    const SmemLayout L = smem_layout(4, 1, 0, 1, 1, false, false, 0, -1, 0);
+    const int n = A.n, m = A.m, T = A.t_max, t_smooth = A.t_smooth, dv_max = A.dv_max, dc8 = (A.dc_max + 7) >> 3;
+    const int groups = (n + 3) >> 2;
+    const long long* lane_frame = reinterpret_cast<const long long*>(smem + L.off_frame);
+    uint32_t* ctl = reinterpret_cast<uint32_t*>(smem + L.off_ctl);
+    uint32_t* tally = reinterpret_cast<uint32_t*>(smem + L.off_best);
+    const uint4* keys = reinterpret_cast<const uint4*>(tally + 4);
+    const float4* icdf = reinterpret_cast<const float4*>(smem + off_icdf);
+    uint32_t* xw = reinterpret_cast<uint32_t*>(smem + off_xw);
+    uint4* xw4 = reinterpret_cast<uint4*>(xw);
+    uint32_t* sw = reinterpret_cast<uint32_t*>(smem + off_sw);
+    uint4* cnt = reinterpret_cast<uint4*>(smem + off_cnt);
+    const uint32_t* thr = reinterpret_cast<const uint32_t*>(smem + off_thr);
+    uint16_t* st = ST_SMEM ? reinterpret_cast<uint16_t*>(smem + off_st) : st_cta;
+    const uint32_t* deg4 = reinterpret_cast<const uint32_t*>(sym_deg);
+    const uint2* units = reinterpret_cast<const uint2*>(sym_chks);
+    const int tid = threadIdx.x, lane = tid & 31, nwarps = blockDim.x >> 5, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    const uint32_t live = ctl[2];
+    const bool act = (live >> lane) & 1u;
+    auto job_of = [&](int f) -> const Job& { return CHAIN ? jl[slot_e[f]] : A; };
+    const float scale = job_of(lane).scale;
+    const uint64_t frame = job_of(lane).frame_offset + (uint64_t)(act ? lane_frame[lane] : 0);
+    const int start = reinterpret_cast<const int32_t*>(smem + L.off_start)[lane];
+    const uint32_t* cntw = reinterpret_cast<const uint32_t*>(cnt) + cnt_word(lane);
+    const int csh = cnt_shift(lane);
+    const bool uniform = A.uniform != 0;
+    const MetricConsts M = {A.w, A.fix_R, A.fix_kmax, A.fix_W, A.acc_R, A.acc_W};
+    const int seen = (int)tally[0], most = groups * kFullMarks;
+
+    // the slots' held samples
+    for (int k = tid; k < n; k += blockDim.x)
+        for (uint32_t r = live; r; r &= r - 1u) {
+            const int f = __ffs(r) - 1;
+            const Job& Jf = job_of(f);
+            ys[gidx(k, f)] = hold<PREC>(read_sample(Jf, lane_frame[f], k), Jf);
+        }
+    if (tid == 0) tally[1] = tally[2] = 0u;
+    __syncthreads();
+
+    uint32_t fin = 0u;
+    int least = -1;                     // flips below which it ends (-1: none counted yet)
+    for (;;) {
+        ++round;
+        // ---- A. syndromes (two threads XOR half of a check each) and the vote ----
+        uint32_t acc = 0u;
+        if (tid == 0) ctl[(round + 1) & 1] = 0u;
+        const int h = tid & 1;
+        const uint2* cols = reinterpret_cast<const uint2*>(chk_cols);
+        for (int base = 0; base < m; base += blockDim.x >> 1) {
+            const int i = base + (tid >> 1);
+            uint32_t s = 0u;
+            if (i < m) {
+#pragma unroll 2
+                for (int v = 0; v < dc8; ++v) {
+                    const uint2 c = cols[2 * (v * m + i) + h];
+                    s ^= xw[c.x & 0xFFFFu] ^ xw[c.x >> 16];
+                    s ^= xw[c.y & 0xFFFFu] ^ xw[c.y >> 16];
+                }
+            }
+            s ^= __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+            if (i < m) sw[2 * i + h] = spread_pairs((s >> (16 * h)) & 0xFFFFu);
+            acc |= s;
+        }
+        acc = __reduce_or_sync(0xFFFFFFFFu, acc);
+        if (lane == 0 && acc) atomicOr(ctl + (round & 1), acc);
+        __syncthreads();
+        const int t = act ? round - start : 0;
+        fin = live & (~ctl[round & 1] | __ballot_sync(0xFFFFFFFFu, act && t >= T));
+        if (fin) break;
+        // (every thread has read the flips of the last iteration, whose word this is)
+        if (tid == 0) tally[1 + ((round + 1) & 1)] = 0u;
+        // ---- A'. counts of unsatisfied checks ----
+        count_groups(cnt, sw, groups, dv_max, [&](int i, int e, int d) { return units[(size_t)(e + d) * sym_groups + (i >> 1)]; });
+        __syncthreads();
+        // ---- C. Step 2 and Step 3b for every symbol of every live slot, two groups at a time ----
+        unsigned flipped = 0;
+        PhiloxKeys G;
+        {
+            const uint4 k0 = keys[0];
+            G.rk0[0] = k0.x; G.rk1[0] = k0.y; G.rk0[1] = k0.z; G.rk1[1] = k0.w;
+        }
+        const PhiloxLane ph(frame, (uint32_t)t, G);
+        for (int g0 = 2 * warp; g0 < groups; g0 += 2 * nwarps) {
+            const bool two = g0 + 1 < groups;
+            const int gs[2] = {g0, two ? g0 + 1 : g0};      // (a single last group twice, once without effect)
+            typename Held<PREC>::T yv[2][4];
+            [[maybe_unused]] uint2 sv[2];
+            uint32_t s4[2], rnd[2][4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int at = (gs[u] * kSlots + lane) * 4;         // this lane's entries in the group layout
+                load_held4(ys + at, yv[u]);
+                if constexpr (kState) sv[u] = *reinterpret_cast<const uint2*>(st + at);
+                // S_k + 64, a byte each
+                s4[u] = deg4[gs[u]] + 0x40404040u - 2u * ((cntw[16 * gs[u]] >> csh) & 0x0F0F0F0Fu);
+            }
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {
+                const uint4 q = keys[r];
+                G.rk0[2 * r] = q.x; G.rk1[2 * r] = q.y; G.rk0[2 * r + 1] = q.z; G.rk1[2 * r + 1] = q.w;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) ph.group((uint32_t)gs[u], G, rnd[u]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int at = (gs[u] * kSlots + lane) * 4;
+                const int have = n - 4 * gs[u];     // (the missing symbols of a partial last group keep their zeros)
+                const uint4 x4 = xw4[gs[u]];
+                uint32_t fmv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t word = j == 0 ? x4.x : j == 1 ? x4.y : j == 2 ? x4.z : x4.w;
+                    const uint32_t xsign = (word << (31 - lane)) & 0x80000000u;
+                    const float z = uniform ? uniform_dev(rnd[u][j]) : gauss_icdf(rnd[u][j], icdf);
+                    typename Metric<PREC>::T S;
+                    // (a byte in the mantissa of 2^23: no conversion instruction)
+                    if constexpr (PREC == kFP32 || PREC == kFP16) S = __uint_as_float(__byte_perm(s4[u], 0x4B000000u, 0x7540 + j)) - 8388672.0f;
+                    else S = (int)((s4[u] >> (8 * j)) & 0xFFu) - 64;
+                    const auto E = metric<PREC>(yv[u][j], xsign, S, __fmul_rn(scale, z), M);
+                    [[maybe_unused]] uint32_t s0 = 0u;
+                    if constexpr (kState) s0 = j < 2 ? (sv[u].x >> (16 * j)) & 0xFFFFu : (sv[u].y >> (16 * (j - 2))) & 0xFFFFu;
+                    const uint32_t th = ADAPT ? thr[(t - (int)(s0 & kUMask)) & kUMask] : th0;
+                    const bool flip = below<PREC>(E, th) && act && (u == 0 || two) && (j == 0 || j < have);
+                    flipped += flip ? 1u : 0u;
+                    if constexpr (kState) {
+                        if (flip) st[at + j] = (uint16_t)flipped_state<ADAPT, SMOOTH>(s0, xsign != 0u, t, T, t_smooth);
+                    }
+                    fmv[j] = __ballot_sync(0xFFFFFFFFu, flip);
+                }
+                if (lane == 0 && (u == 0 || two))
+                    xw4[gs[u]] = make_uint4(x4.x ^ fmv[0], x4.y ^ fmv[1], x4.z ^ fmv[2], x4.w ^ fmv[3]);
+            }
+        }
+        flipped = __reduce_add_sync(0xFFFFFFFFu, flipped);
+        if (lane == 0 && flipped) atomicAdd(tally + 1 + (round & 1), flipped);
+        __syncthreads();
+        // (the flips of the first iteration stand for the outputs evaluated in the one before)
+        const int now = (int)tally[1 + (round & 1)];
+        if (least < 0) least = (int)(7ll * now * most / (8ll * seen));
+        if (now < least) {
+            ++round;
+            break;
+        }
+    }
+    // ---- the margins of the slots that go on, and of the missing symbols of a partial last group ----
+    uint8_t* yb = reinterpret_cast<uint8_t*>(ys);
+    __syncthreads();
+    if (tid < 2) ctl[tid] = ctl[6 + tid] = 0u;
+    for (int k = tid; k < pad4(n); k += blockDim.x) {
+        const uint32_t word = k < n ? xw[k] : 0u;
+        if (k >= n)
+            for (int f = 0; f < kSlots; ++f) yb[gidx(k, f)] = (uint8_t)(int)A.pf_hi;
+        else
+            for (uint32_t r = live & ~fin; r; r &= r - 1u) {
+                const int f = __ffs(r) - 1;
+                const Job& Jf = job_of(f);
+                yb[gidx(k, f)] = (uint8_t)margin_byte<PREC>(hold<PREC>(read_sample(Jf, lane_frame[f], k), Jf),
+                                                            ((word >> f) & 1u) << 31, sym_deg[k], Jf);
+            }
+    }
+    __syncthreads();
+    return round;
 }
 
 // The slot loop for one job (rows a0-a8 of the method): CTA-wide, returns when the job
@@ -862,7 +1111,11 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
     // threshold of the non-adaptive variants; chained jobs read it once here, since the first
     // job's memory is returned when that job completes
     const uint32_t th0_once = CHAIN ? __ldcg(thr_src) : 0u;
-    if (tid < (CHAIN ? 1 : 2) * kSlots) best[tid] = ~0ull;
+    // not single-bit: the outputs evaluated in an iteration, the flips of one of full_rounds (two, by
+    // parity), and at 16 bytes the generator's round keys for it
+    uint32_t* tally = reinterpret_cast<uint32_t*>(best);
+    if (tid < (CHAIN ? 1 : 2) * kSlots)
+        best[tid] = single ? ~0ull : tid >= 2 && tid < 12 ? (unsigned long long)G.rk1[tid - 2] << 32 | G.rk0[tid - 2] : 0ull;
     if (split) {
         group_sync();        // every copy cleared before rank 0 writes the slot table
         if (tid == 0 && S.rank == 0) {
@@ -1118,6 +1371,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         // ---- A'. per symbol and slot, the count of unsatisfied checks in M(k) ----
         uint32_t* n_flips = ctl + 6 + (round & 1);
         if (tid == 0) ctl[6 + ((round + 1) & 1)] = 0u;
+        if (!WIDE && !single && tid == 0 && (round & kFullEvery) == kFullEvery - 1) tally[0] = 0u;
         if (anew) {
         // a CTA of a split job flips decisions in every copy during phase C: none before every
         // CTA has formed its syndromes (the barrier's wait is below, after the counts)
@@ -1125,38 +1379,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (split) cooperative_groups::this_cluster().barrier_arrive();
         }
         if constexpr (!WIDE) {
-            // two threads per group, each for 16 slots: the four symbols' check words added in
-            // 2-bit lanes three at a time, widened to nibbles (even and odd slots), and the
-            // bytes of the four symbols gathered into the words that phase C reads
-            for (int i = tid; i < 2 * groups_l; i += blockDim.x) {
-                const int gl = i >> 1, h = i & 1;
-                uint32_t ev[4] = {0u, 0u, 0u, 0u}, od[4] = {0u, 0u, 0u, 0u};
-                for (int e = 0; e < dv_max; e += 3) {
-                    uint32_t a[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        if (e + d >= dv_max) break;
-                        const uint2 c = i == tid && e == 0 ? pre[d] : units[(size_t)(e + d) * sym_groups + gl];
-                        a[0] += sw[2 * (c.x & 0xFFFFu) + h];
-                        a[1] += sw[2 * (c.x >> 16) + h];
-                        a[2] += sw[2 * (c.y & 0xFFFFu) + h];
-                        a[3] += sw[2 * (c.y >> 16) + h];
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        ev[j] += a[j] & 0x33333333u;
-                        od[j] += (a[j] >> 2) & 0x33333333u;
-                    }
-                }
-                auto bytes = [](const uint32_t w[4]) {      // word b: byte b of w[0..3]
-                    const uint32_t t0 = __byte_perm(w[0], w[1], 0x5140), t1 = __byte_perm(w[0], w[1], 0x7362);
-                    const uint32_t u0 = __byte_perm(w[2], w[3], 0x5140), u1 = __byte_perm(w[2], w[3], 0x7362);
-                    return make_uint4(__byte_perm(t0, u0, 0x5410), __byte_perm(t0, u0, 0x7632),
-                                      __byte_perm(t1, u1, 0x5410), __byte_perm(t1, u1, 0x7632));
-                };
-                cnt[4 * gl + 2 * h] = bytes(ev);
-                cnt[4 * gl + 2 * h + 1] = bytes(od);
-            }
+            count_groups(cnt, sw, groups_l, dv_max, [&](int i, int e, int d) {
+                return i == tid && e == 0 ? pre[d] : units[(size_t)(e + d) * sym_groups + (i >> 1)];
+            });
         } else {
             for (int k = k_lo + tid; k < k_hi; k += blockDim.x) {
                 const int kk = k - k_lo;                      // local index of the symbol
@@ -1187,15 +1412,9 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         const uint32_t* cntw = reinterpret_cast<const uint32_t*>(cnt);
         const bool uniform = A.uniform != 0;
 
-        // A flip of (symbol kl of this CTA, slot f) at the slot's iteration t: the flip count, and
-        // the window count, which takes the new decision for x(t + 1) .. x(T)
-        auto flipped_state = [&](uint32_t s0, bool was_neg, int t) -> uint32_t {
-            uint32_t s1 = s0 + (ADAPT ? 1u : 0u);
-            if constexpr (SMOOTH) {
-                const uint32_t rem = (uint32_t)(T - max(t + 1, A.t_smooth) + 1) << kCShift;
-                s1 = was_neg ? s1 - rem : s1 + rem;
-            }
-            return s1;
+        // A flip of (symbol kl of this CTA, slot f) at the slot's iteration t
+        auto flip_at = [&](uint32_t s0, bool was_neg, int t) -> uint32_t {
+            return flipped_state<ADAPT, SMOOTH>(s0, was_neg, t, T, A.t_smooth);
         };
 
         // E_k as an order-preserving key and, from the key, in real units (single-bit variant)
@@ -1238,7 +1457,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             const uint32_t csh = (uint32_t)cnt_shift(slot);
             // queue: local group | slot << 16 | outputs at or below their cutoffs << 24
             uint32_t* queue = reinterpret_cast<uint32_t*>(smem + L.off_queue) + warp * kQueue;
-            int queued = 0;
+            int queued = 0, evaluated = 0;
 
             // the exact form for one output of one symbol per lane that is `on`: E_k, its flip (or, in the
             // single-bit variant, its claim to be the slot's least)
@@ -1270,17 +1489,17 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                                 for (int r = 0; split && r < S.size; ++r)
                                     if (r != S.rank) atomicXor(peer(xw, r) + k, 1u << f);
                             }
-                            if constexpr (kState) st[at] = (uint16_t)flipped_state(s0, xsign != 0u, tf);
+                            if constexpr (kState) st[at] = (uint16_t)flip_at(s0, xsign != 0u, tf);
                             yb[at] = (uint8_t)margin_byte<PREC>(h, xsign ^ 0x80000000u, deg, Jf);
                         }
                     }
                 }
-                // recorded while they are few enough to be used (D); one lane reads the count for the
-                // warp, since other warps add to it meanwhile
+                // recorded while they are few enough to be used (D); the warp takes one lane's reading of
+                // the count, since other warps add to it meanwhile
                 const uint32_t fl = __ballot_sync(0xFFFFFFFFu, flip);
-                if (fl && record) {
-                    int at = kFlips;
-                    if (lane == 0 && *(volatile uint32_t*)n_flips <= (uint32_t)few) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
+                if (fl && record && __shfl_sync(0xFFFFFFFFu, *(volatile uint32_t*)n_flips, 0) <= (uint32_t)few) {
+                    int at = 0;
+                    if (lane == 0) at = (int)atomicAdd(n_flips, (unsigned)__popc(fl));
                     at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(fl & ((1u << lane) - 1u));
                     if (flip && at < kFlips) flips[at] = (uint32_t)kl | ((uint32_t)f << 16);
                 }
@@ -1290,6 +1509,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             // the draw kept in the sweep); groups with further marks go back into the queue
             auto evaluate = [&](int count) {
                 __syncwarp();
+                evaluated += count;
                 queued -= count;
                 const uint32_t q = lane < count ? queue[queued + lane] : 0u;
                 const int f = q ? (int)((q >> 16) & 31u) : slot, j = (__ffs(q >> 24) - 1) & 3, g = (int)(q & 0xFFFFu);
@@ -1380,6 +1600,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (lg == 5) run(std::true_type{});
             else run(std::false_type{});
             while (queued) evaluate(queued < 32 ? queued : 32);
+            if (!single && (round & kFullEvery) == kFullEvery && lane == 0 && evaluated) atomicAdd(tally, (unsigned)evaluated);
         } else {
             // every symbol of every slot, lane = slot (an idle slot's decisions and counters are
             // don't-care: cleared when it takes a frame, never part of an output)
@@ -1396,12 +1617,11 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 const int at = (gl * kSlots + lane) * 4;  // this lane's entries in the group layout
                 HeldT yv[4];
                 load_held4(ys + at, yv);
-                [[maybe_unused]] uint32_t sv[4] = {0u, 0u, 0u, 0u}, c4 = 0u;
+                [[maybe_unused]] uint32_t sv[4] = {0u, 0u, 0u, 0u};
                 if constexpr (kState) {
                     const uint2 s2 = *reinterpret_cast<const uint2*>(st + at);
                     sv[0] = s2.x & 0xFFFFu; sv[1] = s2.x >> 16; sv[2] = s2.y & 0xFFFFu; sv[3] = s2.y >> 16;
                 }
-                if constexpr (!WIDE) c4 = cntw[16 * gl + cnt_word(lane)] >> cnt_shift(lane);
                 const uint4 x4 = reinterpret_cast<const uint4*>(xw)[g];
                 const uint32_t xwv[4] = {x4.x, x4.y, x4.z, x4.w};
                 float z[4];
@@ -1411,17 +1631,12 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                 for (int j = 0; j < 4; ++j) {
                     const int k = k0 + j;
                     if (k >= k_hi) break;
-                    int Sk;
-                    if constexpr (!WIDE) {
-                        Sk = (int)sym_deg[k - sym_base] - 2 * (int)((c4 >> (8 * j)) & 0xFu);
-                    } else {
-                        const uint4 c = cnt[2 * (k - k_lo)], d = cnt[2 * (k - k_lo) + 1];
-                        const int unsat_cnt = (int)(((c.x >> lane) & 1u) | (((c.y >> lane) & 1u) << 1) |
-                                                    (((c.z >> lane) & 1u) << 2) | (((c.w >> lane) & 1u) << 3) |
-                                                    (((d.x >> lane) & 1u) << 4) | (((d.y >> lane) & 1u) << 5) |
-                                                    (((d.z >> lane) & 1u) << 6));
-                        Sk = (int)d.w - 2 * unsat_cnt;
-                    }
+                    const uint4 c = cnt[2 * (k - k_lo)], d = cnt[2 * (k - k_lo) + 1];
+                    const int unsat_cnt = (int)(((c.x >> lane) & 1u) | (((c.y >> lane) & 1u) << 1) |
+                                                (((c.z >> lane) & 1u) << 2) | (((c.w >> lane) & 1u) << 3) |
+                                                (((d.x >> lane) & 1u) << 4) | (((d.y >> lane) & 1u) << 5) |
+                                                (((d.z >> lane) & 1u) << 6));
+                    const int Sk = (int)d.w - 2 * unsat_cnt;
                     const uint32_t xsign = (xwv[j] << (31 - lane)) & 0x80000000u;
                     const auto E = metric<PREC>(yv[j], xsign, Sk, __fmul_rn(scale, z[j]), A);
                     if (single) {
@@ -1432,7 +1647,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                         const uint32_t th = ADAPT ? thr[(t - (int)(sv[j] & kUMask)) & kUMask] : th0;
                         const bool flip = below<PREC>(E, th);
                         if constexpr (kState) {
-                            if (flip) st[at + j] = (uint16_t)flipped_state(sv[j], xsign != 0u, t);
+                            if (flip) st[at + j] = (uint16_t)flip_at(sv[j], xsign != 0u, t);
                         }
                         fmv[j] = __ballot_sync(0xFFFFFFFFu, flip);
                     }
@@ -1473,7 +1688,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
                     const bool was_neg = (atomicXor(xw + k, 1u << tid) >> tid) & 1u;
                     if (k >= k_lo && k < k_hi) {
                         const int at = gidx(k - k_lo, tid);
-                        if constexpr (SMOOTH) st[at] = (uint16_t)flipped_state(st[at], was_neg, round - lane_start[tid]);
+                        if constexpr (SMOOTH) st[at] = (uint16_t)flip_at(st[at], was_neg, round - lane_start[tid]);
                         if constexpr (!dense) {
                             const Job& Jf = job_of(tid);
                             yb[at] = (uint8_t)margin_byte<PREC>(hold<PREC>(read_sample(Jf, lane_frame[tid], k), Jf),
@@ -1505,6 +1720,13 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         // ---- D. the syndromes and counts moved by the flips, when these are few ----
         anew = true;
         if constexpr (!WIDE) {
+            if (!single && !split && (round & kFullEvery) == kFullEvery && __popc(live) > kSlots / 2 &&
+                tally[0] > (uint32_t)(groups_l * kFullMarks) && A.trace_u == nullptr) {
+                round = full_rounds<ADAPT, SMOOTH, ST_SMEM, PREC, CHAIN>(
+                    A, ch.jl, ch.slot_e, L.off_icdf, L.off_cnt, L.off_xw, L.off_sw, L.off_thr, L.off_st, chk_cols, sym_chks,
+                    sym_deg, sym_groups, ys, st, th0, round);
+                continue;
+            }
             const int nf = record ? (int)*n_flips : 0;
             if (record && nf <= few) {
                 anew = false;

@@ -10,7 +10,7 @@ __global__ void __launch_bounds__(1024) ngdbf_multi_kernel(const __grid_constant
     using HeldT = typename Held<PREC>::T;
     __shared__ Job job;
     __shared__ int32_t next_job;
-    HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, A.n_max);
+    HeldT* ys = slot_scratch<PREC>(A.yslots, blockIdx.x, A.n_max);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_max) * kSlots : nullptr;
     int j = A.first_job[blockIdx.x];
     while (j >= 0) {

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(1024) ngdbf_multi_cluster_kernel(const __grid_
     __shared__ Job job;
     __shared__ int32_t next_job;
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, A.n_local);
+    HeldT* ys = slot_scratch<PREC>(A.yslots, blockIdx.x, A.n_local);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_local) * kSlots : nullptr;
     int j = A.first_job[blockIdx.x / C];
     while (j >= 0) {

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
     Job& job = jl[0];
     int& pick = sh.pick;
     if (threadIdx.x == 0) sh.fail[0] = sh.fail[1] = ~0ull;
-    HeldT* ys = slot_scratch<PREC, WIDE>(A.yslots, blockIdx.x, A.n_max);
+    HeldT* ys = slot_scratch<PREC>(A.yslots, blockIdx.x, A.n_max);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(A.n_max) * kSlots : nullptr;
     const volatile ServeRing* R = A.ring;
     long long slept = 0;
@@ -446,7 +446,7 @@ ngdbf_status plan_serve(ngdbf_server* S, const Kind& K, ServePlan* out) {
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     out->grid = sms * out->sp.bps;
-    out->per_y = (size_t)pad4(K.n) * kSlots * slot_bytes(K.precision, wide);
+    out->per_y = (size_t)pad4(K.n) * kSlots * held_bytes(K.precision);
     out->per_st = (state && !out->sp.st_smem) ? (size_t)pad4(K.n) * kSlots * 2 : 0;
     out->bytes = align256((size_t)out->grid * out->per_y) + align256((size_t)out->grid * out->per_st) + kMarginSlack;
     return NGDBF_OK;
