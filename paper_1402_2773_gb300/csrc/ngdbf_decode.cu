@@ -69,6 +69,9 @@ __global__ void __launch_bounds__(256) mix_probe_kernel(const __grid_constant__ 
     atomicXor(sink, xw[0] ^ xw[1] ^ xw[2] ^ xw[3] ^ sv[0] ^ sv[1] ^ sv[2] ^ sv[3]);
 }
 
+// Frames in the slots of the running launches (Job::in_flight).
+__device__ unsigned int g_in_flight;
+
 template <bool ADAPT, bool SMOOTH, bool ST_SMEM, bool WIDE, int PREC>
 __global__ void __launch_bounds__(1024) ngdbf_persistent_kernel(const __grid_constant__ DecodeArgs A) {
     using HeldT = typename Held<PREC>::T;
@@ -76,6 +79,8 @@ __global__ void __launch_bounds__(1024) ngdbf_persistent_kernel(const __grid_con
     HeldT* ys = slot_scratch<PREC>(A.yslots, blockIdx.x, J.n);
     uint16_t* st = A.st_global ? A.st_global + (size_t)blockIdx.x * pad4(J.n) * kSlots : nullptr;
     decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(J, A.thr, A.G, with_fixed_offsets<WIDE>(A.L), A.placement, ys, st);
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (threadIdx.x == 0) atomicSub(J.in_flight, reinterpret_cast<const uint32_t*>(smem + A.L.off_ctl)[4]);
 }
 
 }  // namespace ngdbf
@@ -234,7 +239,7 @@ void host_gen_consts(uint64_t seed, GenConsts& G) {
 int spread_least(bool wide) { return wide ? kSlots : 1; }
 
 struct LaunchPlan {
-    int block, grid, blocks_per_sm, smem, slots_least;
+    int block, grid, cap, blocks_per_sm, smem, slots_least;
     bool st_smem;
     int placement;              // adjacency tables in shared memory: kTabChk | kTabSym
 };
@@ -393,7 +398,8 @@ ngdbf_status plan_launch(const ngdbf_code* C, const ngdbf_params* P, int64_t n_f
     plan->block = best_block;
     plan->blocks_per_sm = best_bps;
     plan->slots_least = spread_least(wide);
-    plan->grid = (int)std::min<int64_t>((int64_t)sm_count * best_bps, (n_frames + plan->slots_least - 1) / plan->slots_least);
+    plan->cap = sm_count * best_bps;
+    plan->grid = (int)std::min<int64_t>(plan->cap, (n_frames + plan->slots_least - 1) / plan->slots_least);
     plan->smem = L.total;
     plan->st_smem = st_smem;
     plan->placement = placement;
@@ -526,6 +532,20 @@ void fill_job(const ngdbf_code* C, const ngdbf_params* P, const float* y, int64_
     fill_margins(C, P, thr, &J);
 }
 
+// Address of g_in_flight on a device (the current one).
+ngdbf_status in_flight_word(int dev, unsigned int** out) {
+    static std::mutex mu;
+    static void* addr[64] = {};
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev < 0 || dev >= 64) return fail(NGDBF_ERR_UNSUPPORTED, "device index out of range");
+    if (!addr[dev]) {
+        cudaError_t e = cudaGetSymbolAddress(&addr[dev], g_in_flight);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
+    }
+    *out = static_cast<unsigned int*>(addr[dev]);
+    return NGDBF_OK;
+}
+
 // Frames a CTA takes first when n_frames are decoded by n_ctas CTAs, `least` at least (spread_least).
 int first_slots(int64_t n_frames, int64_t n_ctas, int least) {
     const int64_t per = (n_frames + n_ctas - 1) / std::max<int64_t>(n_ctas, 1);
@@ -534,7 +554,7 @@ int first_slots(int64_t n_frames, int64_t n_ctas, int least) {
 
 // Kernel arguments of one decode: scratch at `base` (work counter, then the
 // per-slot samples), per-slot state at `st_base` when it lives in global memory.
-void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& plan, int grid, const float* y,
+void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& plan, int grid, unsigned int* in_flight, const float* y,
                int64_t n_frames, float sigma, uint64_t seed, uint64_t frame_offset, uint8_t* bits,
                int32_t* iters, uint8_t* pass, unsigned char* base, unsigned char* st_base,
                bool st_global, DecodeArgs* out) {
@@ -544,6 +564,8 @@ void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& pla
              reinterpret_cast<unsigned long long*>(base), &A.J, A.thr);
     A.J.thr = nullptr;                 // thresholds travel inline in the launch
     A.J.slots = first_slots(n_frames, grid, plan.slots_least);
+    A.J.in_flight = in_flight;
+    A.J.cap = plan.cap;
     A.placement = plan.placement;
     A.L = smem_layout(C->n, C->m, P->t_max, C->dv_max, C->dc_max, (P->variant & NGDBF_ADAPT) != 0,
                       plan.st_smem && (P->variant & 3) != 0, plan.placement);
@@ -621,6 +643,9 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count);
     if (s != NGDBF_OK) return s;
 
+    unsigned int* in_flight = nullptr;
+    s = in_flight_word(dev, &in_flight);
+    if (s != NGDBF_OK) return s;
     cudaMemPool_t pool;
     s = get_pool(dev, &pool);
     if (s != NGDBF_OK) return s;
@@ -651,7 +676,7 @@ ngdbf_status decode_impl(const ngdbf_code* C, const float* y, int64_t n_frames, 
     unsigned char* base = static_cast<unsigned char*>(ws);
 
     DecodeArgs A;
-    fill_args(C, P, plan, plan.grid, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
+    fill_args(C, P, plan, plan.grid, in_flight, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
               base + 256 + bytes_y, bytes_st != 0, &A);
     if (tr && tr->frames > 0) {
         A.J.trace_u = tr->unsat;
@@ -1022,6 +1047,9 @@ extern "C" ngdbf_status ngdbf_decode_noalloc(const ngdbf_code_t* C, const float*
     s = plan_launch(C, P, n_frames, dev, &plan, &fn, &sm_count, true);
     if (s != NGDBF_OK) return s;
 
+    unsigned int* in_flight = nullptr;
+    s = in_flight_word(dev, &in_flight);
+    if (s != NGDBF_OK) return s;
     // Fit the launch into the static array: fewer CTAs when a full grid does not fit.
     const bool state = (P->variant & 3) != 0;
     const size_t per_cta_y = (size_t)pad4(C->n) * kSlots * held_bytes(P->precision);
@@ -1036,7 +1064,7 @@ extern "C" ngdbf_status ngdbf_decode_noalloc(const ngdbf_code_t* C, const float*
     const size_t bytes_y = ((size_t)grid * per_cta_y + 255) / 256 * 256;
 
     DecodeArgs A;
-    fill_args(C, P, plan, grid, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
+    fill_args(C, P, plan, grid, in_flight, y, n_frames, sigma, seed, frame_offset, bits, iters, pass, base,
               base + 256 + bytes_y, per_cta_st != 0, &A);
     // The work counter must start at zero; the kernel initializes everything else it reads.
     e = cudaMemsetAsync(A.J.queue, 0, sizeof(unsigned long long), stream);
