@@ -324,10 +324,10 @@ ngdbf_status choose_placement(int dev, int n, int m, int t_max, int dv_max, int 
         for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0, kTight}) {
             // only where nothing else fits
             if (tb == kTight && (best.bps > 0 || st || dv_max > kNarrowDegree || (use > kTable && u == use))) continue;
-            const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, -1, -1, u);
-            if (L.total > limit) continue;
             for (const int block : {1024, 512, 256, kTightThreads}) {
-                if ((tb == kTight) != (block == kTightThreads)) continue;
+                if (block == kTightThreads && tb != kTight) continue;
+                const SmemLayout L = smem_layout(n, m, t_max, dv_max, dc_max, adapt, st, tb, -1, -1, u, block / 32);
+                if (L.total > limit) continue;
                 int bps = 0;
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, block, L.total);
                 if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
@@ -568,7 +568,7 @@ void fill_args(const ngdbf_code* C, const ngdbf_params* P, const LaunchPlan& pla
     A.J.cap = plan.cap;
     A.placement = plan.placement;
     A.L = smem_layout(C->n, C->m, P->t_max, C->dv_max, C->dc_max, (P->variant & NGDBF_ADAPT) != 0,
-                      plan.st_smem && (P->variant & 3) != 0, plan.placement);
+                      plan.st_smem && (P->variant & 3) != 0, plan.placement, -1, -1, kLaunch, plan.block / 32);
     A.yslots = base + 256;
     A.st_global = st_global ? reinterpret_cast<uint16_t*>(st_base) : nullptr;
     host_gen_consts(seed, A.G);
@@ -1164,7 +1164,7 @@ std::vector<int32_t> assign_ctas_capped(const std::vector<int64_t>& frames, cons
 // of the `tables` as fit in `limit`; -1 when some job does not fit at all.  With a cluster of
 // C > 1 CTAs, jobs of at least split_min_n symbols hold their share of the symbols per CTA.
 int table_smem(const ngdbf_job* jobs, int32_t n_jobs, int C, int split_min_n, bool adapt, bool st, bool wide,
-               int tables, int limit, bool* tight = nullptr) {
+               int tables, int limit, bool* tight = nullptr, int warps = 0) {
     int total = 0;
     if (tight) *tight = false;
     for (int j = 0; j < n_jobs; ++j) {
@@ -1172,7 +1172,7 @@ int table_smem(const ngdbf_job* jobs, int32_t n_jobs, int C, int split_min_n, bo
         const int n_local = (C > 1 && c->n >= split_min_n) ? split_local_max(c->n, C) : c->n;
         int tb = 0;
         const SmemLayout L = job_layout(c->n, c->m, jobs[j].params.t_max, c->dv_max, c->dc_max, adapt, st, wide,
-                                        tables, n_local, limit, &tb);
+                                        tables, n_local, limit, &tb, kTable, warps);
         if (L.total > limit || ((tb & kTight) && !tight)) return -1;
         if (tb & kTight) *tight = true;
         total = std::max(total, L.total);
@@ -1223,11 +1223,10 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         for (const int tb : {kTabChk | kTabSym, kTabChk, kTabSym, 0}) {
-            bool tight = false;         // some job needs the tight layout: its block size for all
-            const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, st, T.wide, tb, limit, &tight);
-            if (total < 0) continue;
             for (const int block : {1024, 512, 256, kTightThreads}) {
-                if (tight != (block == kTightThreads)) continue;
+                bool tight = false;         // some job needs the tight layout: its block size for all
+                const int total = table_smem(jobs, n_jobs, 1, INT32_MAX, adapt, st, T.wide, tb, limit, &tight, block / 32);
+                if (total < 0 || (block == kTightThreads && !tight)) continue;
                 int bps = 0;
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)fn, block, total);
                 if (e != cudaSuccess) return cuda_fail(e, "occupancy");
@@ -1239,7 +1238,7 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
                     T.smem = total;
                     T.st_smem = st;
                     T.placement = tb;
-                    T.tight = tight;
+                    T.tight_block = tight ? block : 0;
                 }
             }
         }
@@ -1247,7 +1246,7 @@ ngdbf_status plan_table(const ngdbf_job* jobs, int32_t n_jobs, int dev, TablePla
     if (best_bps == 0) return fail(NGDBF_ERR_UNSUPPORTED, "code too large for the shared-memory decision words");
     T.state_global = state && !T.st_smem;
     for (int block : {1024, 512, 256, kTightThreads}) {
-        if (T.tight != (block == kTightThreads)) continue;
+        if (T.tight_block ? block != T.tight_block : block == kTightThreads) continue;
         int bps = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)T.fn, block, T.smem);
         if (e != cudaSuccess) return cuda_fail(e, "occupancy");

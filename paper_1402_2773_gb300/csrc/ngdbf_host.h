@@ -58,7 +58,7 @@ struct TablePlan {
     int n_max = 0, m_max = 0, t_max = 0, dv_max = 0, dc_max = 0;
     int variant = 0, precision = 0, sm_count = 0, smem = 0;
     bool st_smem = false, wide = false, state_global = false;
-    bool tight = false;         // some job is laid out with kTight: blocks of kTightThreads
+    int tight_block = 0;        // some job is laid out with kTight: the only block size
     int placement = 0;          // adjacency tables in shared memory: kTabChk | kTabSym
     size_t thr_words = 0;
     void* fn = nullptr;

@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(1024) ngdbf_multi_kernel(const __grid_constant
         int tables = 0;
         const SmemLayout L = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT,
                                         ST_SMEM && (ADAPT || SMOOTH), WIDE, A.placement, job.n, A.smem_bytes,
-                                        &tables);
+                                        &tables, kTable, blockDim.x >> 5);
         decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC>(job, job.thr, A.G, L, tables, ys, st);
         // the next job: the one with the most unclaimed work (none left: done)
         if (threadIdx.x == 0) {

@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
         bool done = false;
         if constexpr (kState && !ST_SMEM && !WIDE) {
             const SmemLayout Ls = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT, true, WIDE,
-                                             A.placement, job.n, A.smem_bytes, &tables, kServe);
+                                             A.placement, job.n, A.smem_bytes, &tables, kServe, blockDim.x >> 5);
             if (Ls.total <= A.smem_bytes) {
                 ch.entries = Ls.cuts;
                 decode_job<ADAPT, SMOOTH, true, WIDE, PREC, false, true, RingNext>(
@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(1024) ngdbf_serve_kernel(const __grid_constant
         if (!done) {
             // (a code no larger than the kind's maxima always fits without its state)
             const SmemLayout L = job_layout(job.n, job.m, job.t_max, job.dv_max, job.dc_max, ADAPT,
-                                            ST_SMEM && kState, WIDE, A.placement, job.n, A.smem_bytes, &tables, kServe);
+                                            ST_SMEM && kState, WIDE, A.placement, job.n, A.smem_bytes, &tables, kServe,
+                                            blockDim.x >> 5);
             if constexpr (!WIDE) ch.entries = L.cuts;
             decode_job<ADAPT, SMOOTH, ST_SMEM, WIDE, PREC, false, true, RingNext>(
                 job, job.thr, A.G, with_fixed_offsets<WIDE, kServe>(L), tables, ys, st, Split{0, 1, 0, 0}, ch);

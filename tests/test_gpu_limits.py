@@ -98,3 +98,20 @@ def test_codes_whose_maxima_do_not_fit_together(O):
     for got, ref in zip(outs, want):
         for a, b in zip(got, ref):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,m,block", [(11000, 172, 256), (10950, 300, 512), (10600, 700, 1024)])
+def test_threads_of_the_longest_codes(O, n, m, block):
+    """As many warps as there are syndrome words for their queues."""
+    code = long_code(n, m)
+    gp, op = params_pair(variant=3, lam=0.95, t_max=8, smooth_window=3, w=0.4, theta=-0.5)
+    y, _, _ = wl.frames(code, 152 * 3, None, seed=5, sigma=0.8)
+    dc = ngdbf.DeviceCode.from_code(code)
+    try:
+        got = dc.decode(torch.from_numpy(y).cuda(), 0.8, gp, seed=2)
+        torch.cuda.synchronize()
+        assert ngdbf.ngdbf_last_launch()["block"] == block
+    finally:
+        dc.close()
+    for a, b in zip(got, O.decode_f32(code, y, 0.8, op, seed=2, threads=THREADS)):
+        assert np.array_equal(a.cpu().numpy(), b)

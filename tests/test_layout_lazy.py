@@ -37,7 +37,7 @@ struct Span { const char* name; int at, bytes; };
 
 // Every array of L with the bytes the kernel uses of it.
 static bool sane(const SmemLayout& L, int n, int m, int nl, int dv, int dc, bool thr, bool st, int tables, bool wide,
-                 int use) {
+                 int use, int warps) {
     const bool serve = use > kTable, tight = tables & kTight;
     Span a[] = {{"frame", L.off_frame, kSlots * 8}, {"start", L.off_start, kSlots * 4}, {"ctl", L.off_ctl, 32},
                 {"unsat", wide ? -1 : L.off_unsat, kSlots * 4}, {"best", L.off_best, (serve ? 1 : 2) * kSlots * 8},
@@ -65,7 +65,7 @@ static bool sane(const SmemLayout& L, int n, int m, int nl, int dv, int dc, bool
     if ((thr && L.off_thr < 0) || (st && L.off_st < 0)) { printf("FAIL thr or state\n"); return false; }
     if (!wide && L.off_cnt + pad4(nl) * 16 + 31 * 64 > L.total) { printf("FAIL counts read past the total\n"); return false; }
     const int end = thr ? L.off_thr : L.total;
-    if (tight && (L.off_queue != L.off_sw || L.off_flips != -1 || st || wide || end - L.off_sw < kTightThreads / 32 * kQueue * 4)) { printf("FAIL tight\n"); return false; }
+    if (tight && (L.off_queue != L.off_sw || L.off_flips != -1 || st || wide || end - L.off_sw < warps * kQueue * 4)) { printf("FAIL tight\n"); return false; }
     return L.total % 16 == 0;
 }
 
@@ -74,17 +74,17 @@ static int random_layouts(int cases) {
     for (int c = 0; c < cases; ++c) {
         const bool wide = rnd() % 3 == 0, adapt = rnd() & 1, st = rnd() & 1, serve = rnd() & 1;
         const int use = serve ? kServe : kTable;
-        const int n = in(500, 12000), m = in(std::max(4, n / 64), n), dv = wide ? in(16, 64) : in(1, 15), dc = in(2, 64), P = in(0, 3);
+        const int n = in(500, 12000), m = in(std::max(4, n / 64), n), dv = wide ? in(16, 64) : in(1, 15), dc = in(2, 64), P = in(0, 3), warps = 4 << in(0, 3);
         const SmemLayout A = smem_layout(n, m, 100, dv, dc, adapt, st, P);
-        if (!sane(A, n, m, n, dv, dc, adapt, st, P, dv > kNarrowDegree, kLaunch)) return 1;
+        if (!sane(A, n, m, n, dv, dc, adapt, st, P, dv > kNarrowDegree, kLaunch, warps)) return 1;
         if (!st && dv <= kNarrowDegree && n >= 500) {
-            const SmemLayout B = smem_layout(n, m, 100, dv, dc, adapt, false, kTight);
-            if (!sane(B, n, m, n, dv, dc, adapt, false, kTight, false, kLaunch)) return 1;
+            const SmemLayout B = smem_layout(n, m, 100, dv, dc, adapt, false, kTight, -1, -1, kLaunch, warps);
+            if (!sane(B, n, m, n, dv, dc, adapt, false, kTight, false, kLaunch, warps)) return 1;
         }
         const int C = 1 << in(0, 3), nl = C > 1 && !serve ? split_local_max(n, C) : n, bytes = in(30000, 232448);
         int tb = -1;
-        const SmemLayout J = job_layout(n, m, 100, dv, dc, adapt, st, wide, P, nl, bytes, &tb, use);
-        if (!sane(J, n, m, nl, dv, dc, adapt, st, tb, wide, use)) return 1;
+        const SmemLayout J = job_layout(n, m, 100, dv, dc, adapt, st, wide, P, nl, bytes, &tb, use, warps);
+        if (!sane(J, n, m, nl, dv, dc, adapt, st, tb, wide, use, warps)) return 1;
         if ((tb & ~(P | kTight)) || ((tb & kTight) && (st || wide))) { printf("FAIL placement %d of %d\n", tb, P); return 1; }
         if (serve && !wide && (J.cuts < 1 || J.cuts > kChain || (st && J.total <= bytes && J.cuts != kChain))) {
             printf("FAIL %d cutoff tables\n", J.cuts);
@@ -96,9 +96,9 @@ static int random_layouts(int cases) {
             // a job no larger fits as well, whatever the tables
             const int n2 = in(std::max(8, n / 2), n), m2 = in(std::max(4, n2 / 64), std::max(std::max(4, n2 / 64), std::min(m, n2)));
             if (C == 1 && m2 <= m) {
-                const SmemLayout S = job_layout(n2, m2, 100, dv, dc, adapt, st, wide, P, n2, J.total, &tb, use);
+                const SmemLayout S = job_layout(n2, m2, 100, dv, dc, adapt, st, wide, P, n2, J.total, &tb, use, warps);
                 if (S.total > J.total) { printf("FAIL smaller job: %d > %d\n", S.total, J.total); return 1; }
-                if (!sane(S, n2, m2, n2, dv, dc, adapt, st, tb, wide, use)) return 1;
+                if (!sane(S, n2, m2, n2, dv, dc, adapt, st, tb, wide, use, warps)) return 1;
             }
         }
     }
