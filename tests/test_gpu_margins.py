@@ -24,3 +24,19 @@ def test_samples_at_a_large_threshold(O, theta, variant, prec):
     y = (y * rng.choice([1.0, -1.0], size=y.shape, p=[0.9, 0.1])).astype(np.float32)
     assert_parity(O, code, y, 0.32 * ulp, seed=5, variant=variant, lam=0.999, t_max=12, smooth_window=4,
                   w=0.165 * ulp, theta=theta, eta=0.5, y_max=0.0, **prec)
+
+
+@pytest.mark.parametrize("prec", [dict(), dict(precision=ngdbf.NGDBF_FP16)], ids=["fp32", "fp16"])
+@pytest.mark.parametrize("variant", [0, 3, 4, 6])
+@pytest.mark.parametrize("y_max", [0.0, 2.5])
+def test_samples_that_are_not_numbers(O, variant, y_max, prec):
+    """Such a symbol's E_k is evaluated in every iteration and never below a threshold, nor the least of
+    a frame (the single-bit variant; not symbol 0, where the reference decoder starts its search)."""
+    code = wl.peg_code(504, 252, 3, seed=3)
+    y, _, sig = wl.frames(code, 64, 3.0, seed=9)
+    rng = np.random.default_rng(4)
+    at = rng.random(y.shape)
+    at[:, 0] = 1.0
+    y[at < 0.02] = np.nan
+    y[(at >= 0.02) & (at < 0.025)] = -np.inf
+    assert_parity(O, code, y, sig, seed=6, variant=variant, lam=0.97, t_max=30, smooth_window=10, y_max=y_max, **prec)

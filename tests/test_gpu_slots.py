@@ -11,6 +11,7 @@ import pytest
 
 from paper_1402_2773_gb300 import ngdbf, workload as wl
 from test_gpu_parity import O, _gpu, gpu_decode, irregular_code, params_pair, THREADS  # noqa: F401
+from test_z_lazy import PREC
 
 pytestmark = pytest.mark.gpu
 
@@ -42,3 +43,24 @@ def test_flips_about_the_recorded_number(O, theta, variant):
     """32 slots, from a few flips an iteration of a CTA to some hundred: the count passes the limit
     up to which flips are recorded while warps still add theirs."""
     assert_slots(O, FLIPS, 32, 0.55, variant=variant, lam=0.99, t_max=12, smooth_window=4, w=0.5, theta=theta, eta=0.9)
+
+
+SMALL = irregular_code(203, 101, seed=5)
+BASE = dict(lam=0.97, t_max=10, smooth_window=4, w=0.5, theta=-0.7, eta=0.9)
+
+
+@pytest.mark.parametrize("slots", [2, 5, 17, 31, 32])
+@pytest.mark.parametrize("k,variant", list(enumerate([0, 3, 4, 6, 3 | 8])))
+def test_live_slots_per_cta(O, slots, k, variant):
+    """Some more frames than slots, so that slots are refilled at different iterations."""
+    prec = PREC[(k + slots) % 4]
+    assert_slots(O, SMALL, slots, 0.6, rest=77, variant=variant, **BASE, **prec)
+
+
+@pytest.mark.parametrize("variant", [0, 3, 4])
+@pytest.mark.parametrize("kw", [dict(w=1e-3), dict(w=20.0), dict(theta=0.4), dict(eta=0.0), dict(y_max=0.05, w=0.01, theta=-0.02),
+                                dict(theta=-1e6, lam=0.5, y_max=0.0)], ids=lambda d: ",".join(f"{k}={v}" for k, v in d.items()))
+def test_strain_with_full_slots(O, kw, variant):
+    d = dict(BASE)
+    d.update(kw)
+    assert_slots(O, SMALL, 32, 0.6, variant=variant, **d)
