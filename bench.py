@@ -44,39 +44,22 @@ PRECISIONS = {"fp32": (0, 0, "f32"), "fp16": (1, 0, "f16"), "fix8": (3, 8, "i8")
               "fix8-eq9": (2, 8, "i8")}
 DATA_SEED = 2014          # information bits and channel noise
 DECODER_SEED = 1          # Philox key of the perturbation
-# Lane operations that every (symbol, iteration) of a live frame needs: Philox4x32-10 20 (per 4
-# symbols: 10 rounds of two wide multiplies, counted as 4, and 4 XOR), the margin byte's counts
-# taken off 1, the cutoff lookup 1, the comparison 1.  The counts are formed bit-sliced for 32
-# frames at once, and the deviate, E_k and the counters only for the few outputs at or below
-# their cutoffs: neither is counted.
-OPS_PER_SYMBOL_ITER = 23
-# Lane operations per symbol of the same-mix probe (ngdbf_mix_probe), by the same convention:
-# Philox 20 + deviate 13 + perturbation 1 + inversion function 5 + decision bit 1 + threshold,
-# adaptation, window and ballot 4 + the count lane's extraction 1 (the probe has no per-check
-# penalty work: the decode forms those counts bit-sliced, once for 32 slots).
-PROBE_OPS_PER_SYMBOL = 45
-PROBE_GROUPS = 32768
+# Floor of the decode's arithmetic: every (symbol, iteration) of a live frame needs its Philox output.
+# Four outputs take 18 wide (32 x 32 -> 64 bit) multiplies per lane, two of the twenty being shared by a
+# frame's groups, at 1.05 cycles of an SM per warp instruction (measured on GB300, a quarter of the issue
+# rate).  The deviate, E_k and the counters are formed for the few outputs that can flip a symbol, and the
+# check sums for 32 frames at once: neither is counted.
+WIDE_MULTIPLIES = 18
+CYCLES_PER_MULTIPLY = 1.05
 
 
-def mix_probe(ngdbf, stream, reps=5, warmup=2):
-    """Attainable lane-op rate of the dense per-symbol instruction mix (CUDA events, best of reps)."""
-    import torch
-    sink = torch.zeros(1, dtype=torch.int32, device="cuda")
-    threads = 0
-    for _ in range(warmup):
-        threads = ngdbf.ngdbf_mix_probe(PROBE_GROUPS, sink.data_ptr(), stream.cuda_stream)
-    best = None
-    for _ in range(reps):
-        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        a.record(stream)
-        ngdbf.ngdbf_mix_probe(PROBE_GROUPS, sink.data_ptr(), stream.cuda_stream)
-        b.record(stream)
-        b.synchronize()
-        ms = a.elapsed_time(b)
-        best = ms if best is None else min(best, ms)
-    symbols = threads * PROBE_GROUPS * 4
-    return {"lane_op_s": symbols * PROBE_OPS_PER_SYMBOL / (best / 1e3), "ms": best, "threads": threads,
-            "symbols_per_launch": symbols, "ops_per_symbol": PROBE_OPS_PER_SYMBOL}
+def sym_iter_peak(sm_count, mhz):
+    """Symbol-iterations per second at which the generator's multiplies alone fill the SMs."""
+    return sm_count * mhz * 1e6 * 128 / (WIDE_MULTIPLIES * CYCLES_PER_MULTIPLY)
+
+
+PEAK_BASIS = (f"{WIDE_MULTIPLIES} wide multiplies per four symbol-iterations (Philox4x32-10), {CYCLES_PER_MULTIPLY} "
+              "cycles of an SM per warp instruction (measured), at the decode's median SM clock")
 # DRAM bytes (read + write) per decoded frame of the decode kernel from an ncu capture of this
 # workload's mean over the three points; None: captured per point only (13 kB a frame at 4.5 dB,
 # 178 kB at 3.5 dB, where the slots' state and samples of two CTAs per SM exceed L2).
@@ -298,37 +281,19 @@ def run_ours(args):
     fps = frames_total / elapsed
 
     host_outs = [(b.cpu().numpy(), i.cpu().numpy(), p.cpu().numpy()) for b, i, p in outs]
-    with ClockSampler(local) as probe_clk:
-        probe = mix_probe(ngdbf, stream)
-    probe["clocks"] = probe_clk.summary()
     rates = error_rates(code, host_outs, cws)
-    # roofline: algorithmic lane-ops of the iterations the frames needed, per launch
+    # roofline: symbol-iterations the frames needed, per launch, over the generator's floor
     sym_iters = [float(o[1].astype(np.int64).sum()) * code.n for o in host_outs]
     mean_launch_s = float(np.mean(kernel_ms)) / 1e3
-    ops_per_launch = float(np.mean(sym_iters)) * OPS_PER_SYMBOL_ITER
     clocks = clk.summary()
-    peak_mhz = clocks.get("sm_max_mhz") or measured_peaks().get("sm_max_mhz") or 2070.0
-    sm_count = launch.get("sm_count") or 152
-    peak_ops = sm_count * 128 * peak_mhz * 1e6      # 4 schedulers x 32 lanes issue per SM-clock
-    achieved = ops_per_launch / mean_launch_s
+    mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or measured_peaks().get("sm_max_mhz") or 2070.0
+    peak = sym_iter_peak(launch.get("sm_count") or 152, mhz)
+    achieved = float(np.mean(sym_iters)) / mean_launch_s
     # the capture behind DRAM_BYTES_PER_FRAME is of the FP32 kernel
     traffic = DRAM_BYTES_PER_FRAME * F if (DRAM_BYTES_PER_FRAME and args.precision == "fp32") else None
-    # the peak is the measured rate of the same instruction mix (probe), at the probe's clock
-    # scaled to the decode's sampled clock; the nominal issue rate is kept beside it
-    pclk = probe["clocks"].get("sm_mhz") or peak_mhz
-    dclk = clocks.get("sm_mhz") or peak_mhz
-    peak_meas = probe["lane_op_s"] * dclk / pclk
-    rl = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_meas / 1e12, "unit": "Tlane-op/s",
-          "frac": achieved / peak_meas, "traffic": traffic,
-          "peak_basis": f"measured: same-mix probe (ngdbf_mix_probe, {PROBE_OPS_PER_SYMBOL} lane-ops per symbol) "
-                        f"{probe['lane_op_s'] / 1e12:.2f} T at {pclk:.0f} MHz, scaled to the decode's median "
-                        f"{dclk:.0f} MHz",
-          "peak_nominal": peak_ops / 1e12, "frac_nominal": achieved / peak_ops,
-          "peak_nominal_basis": f"{sm_count} SMs x 128 lanes x {peak_mhz:.0f} MHz (max SM clock)",
-          "probe": {k: v for k, v in probe.items() if k != "clocks"} | {"sm_mhz": pclk},
+    rl = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tsymbol-iteration/s",
+          "frac": achieved / peak, "traffic": traffic, "peak_basis": PEAK_BASIS,
           "kernel": "ngdbf_persistent_kernel<ADAPT,SMOOTH>",
-          "ops_per_symbol_iter": OPS_PER_SYMBOL_ITER,
-          "ops_basis": "generator, margin and cutoff of every live symbol-iteration",
           "algorithmic_bytes_per_launch": F * (4 * code.n + nb + 5),
           "traffic_basis": "ncu dram__bytes_read.sum + dram__bytes_write.sum per frame on a 2*10^4-frame "
                            "capture, scaled to the launch's frames" if traffic else
@@ -488,7 +453,6 @@ def run_multicode(args):
         iter_launches = sum(3 * jb["params"]["t_max"] + 3 for jb in jobs)
         t_plain = max_over_ranks(timed(plain), "cuda")
         t_batch = max_over_ranks(timed(lambda: batch.launch(stream)), "cuda")
-        probe = mix_probe(ngdbf, stream)
     same = all(all(torch.equal(a, b) for a, b in zip(o1, o2)) for o1, o2 in zip(batch.outputs, outs))
     same_iter = all(all(torch.equal(a, b) for a, b in zip(o1, o2)) for o1, o2 in zip(batch.outputs, outs_it))
     frames = sum(jb["frames"] for jb in jobs)
@@ -497,17 +461,16 @@ def run_multicode(args):
     fps_iter = frames * args.steps * world / t_iter
     host = [tuple(t.cpu().numpy() for t in o) for o in batch.outputs]
     per_code = []
-    ops = 0.0
+    sym_iters = 0.0
     for jb, o in zip(jobs, host):
         it = o[1].astype(np.int64)
-        ops += float(it.sum()) * jb["code"].n * OPS_PER_SYMBOL_ITER
+        sym_iters += float(it.sum()) * jb["code"].n
         per_code.append({"code": jb["code"].name, "frames": jb["frames"], "ebn0_db": round(jb["ebn0"], 3),
                          "t_max": jb["params"]["t_max"], "avg_iters": float(it.mean()),
                          "pass_rate": float(o[2].mean())})
     clocks = clk.summary()
-    peak_nominal = (launch.get("sm_count") or 152) * 128 * (clocks.get("sm_max_mhz") or 2070.0) * 1e6
-    peak = probe["lane_op_s"]
-    achieved = ops / (t_batch / args.steps)
+    peak = sym_iter_peak(launch.get("sm_count") or 152, clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 2070.0)
+    achieved = sym_iters / (t_batch / args.steps)
     if rank == 0:
         print(json.dumps({
             "metric": "decoded frames/s", "value": fps, "unit": "frames/s", "n_gpus": world,
@@ -529,10 +492,8 @@ def run_multicode(args):
                                "form": "one persistent ngdbf_decode per code"},
             "speedup_vs_plain": fps / fps_plain, "speedup_vs_plain_per_iteration": fps / fps_iter,
             "results_identical": bool(same and same_iter),
-            "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tlane-op/s",
-                         "frac": achieved / peak, "traffic": None,
-                         "peak_basis": f"measured: same-mix probe ({PROBE_OPS_PER_SYMBOL} lane-ops per symbol)",
-                         "peak_nominal": peak_nominal / 1e12, "frac_nominal": achieved / peak_nominal,
+            "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tsymbol-iteration/s",
+                         "frac": achieved / peak, "traffic": None, "peak_basis": PEAK_BASIS,
                          "kernel": "ngdbf_multi_cluster_kernel / ngdbf_multi_kernel (tuned)"},
             "launch": launch, "gpu_launches": args.steps, "clocks": clocks,
         }))
@@ -640,9 +601,9 @@ def run_serving(args):
             lat_s, span_s, stats, outs_s = run_server(trace)
             lat_p, span_p, outs_p = run_plain(trace)
             same = all(all(torch.equal(a, b) for a, b in zip(x, y)) for x, y in zip(outs_s, outs_p))
-            # algorithmic lane operations of the iterations the frames needed (FP32 count)
-            ops = sum(float(o[1].numpy().astype(np.int64).sum()) * codes[c].n * OPS_PER_SYMBOL_ITER
-                      for (_, c, _, _, _, _), o in zip(trace, outs_s))
+            # symbol-iterations the frames needed
+            sym_iters = sum(float(o[1].numpy().astype(np.int64).sum()) * codes[c].n
+                            for (_, c, _, _, _, _), o in zip(trace, outs_s))
             res[label] = {
                 "rate_requests_per_s": rate, "requests": n_req, "frames": frames,
                 "server_frames_per_s": frames / span_s, "server_requests_per_s": n_req / span_s,
@@ -652,11 +613,12 @@ def run_serving(args):
                 "plain_latency_ms": {"p50": float(np.percentile(lat_p, 50)) * 1e3,
                                      "p99": float(np.percentile(lat_p, 99)) * 1e3},
                 "results_identical": bool(same), "server_stats": stats,
-                "server_lane_op_s": ops / span_s}
-        probe = mix_probe(ngdbf, torch.cuda.current_stream())
+                "server_sym_iter_s": sym_iters / span_s}
     clocks = clk.summary()
+    peak = sym_iter_peak(torch.cuda.get_device_properties(0).multi_processor_count,
+                         clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 2070.0)
     for label in res:
-        res[label]["server_alu_frac"] = res[label]["server_lane_op_s"] / probe["lane_op_s"]
+        res[label]["server_alu_frac"] = res[label]["server_sym_iter_s"] / peak
     if rank == 0:
         off = res["offered"]
         print(json.dumps({
