@@ -156,6 +156,8 @@ ngdbf_status ngdbf_code_info(const ngdbf_code_t* code, int32_t* n, int32_t* m,
  * more where the per-slot state is in global memory, for large batches and long
  * codes; and 5 KB) is taken from a library-owned stream-ordered pool
  * and returned on the same stream.  All pointers must be device memory of the current device.
+ * By itself a small batch is spread over every SM; while other such calls have frames
+ * on the device (on other streams), its frames share CTAs.  The results are the same.
  * The decision, syndrome and count words of one CTA's 32 frames must fit the
  * device's shared memory per block (about 20 n + 8 m + 7 KB bytes for symbol
  * degrees up to 15: n up to about 9,300 at rate 1/2 on a 227 KB device); larger
@@ -451,7 +453,7 @@ ngdbf_status ngdbf_gaussian_range(uint32_t start, uint32_t count, float* z, void
 ngdbf_status ngdbf_generator_table(float* out);
 
 /*
- * Same-mix throughput probe (measurement; the paper has no counterpart): every thread of a
+ * Dense-mix throughput probe (measurement; the paper has no counterpart): every thread of a
  * full-occupancy grid runs `groups` steps of the decode's per-slot symbol work for four
  * symbols on register-resident data -- one Philox4x32-10 call, four inverse-CDF deviates
  * (coefficient table in shared memory), the FP32 inversion function from a 4-bit count lane,

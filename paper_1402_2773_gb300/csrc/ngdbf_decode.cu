@@ -29,7 +29,7 @@ __global__ void gaussian_range_kernel(const __grid_constant__ GenConsts G, uint3
         z[i] = gauss_icdf(start + i, tab);
 }
 
-// Same-mix throughput probe: the per-slot work of the decode's symbol loop for `groups` groups of
+// Dense-mix throughput probe: the per-slot work of the dense form's symbol loop for `groups` groups of
 // four symbols on register-resident data (one Philox call, four inverse-CDF deviates from the
 // shared coefficient table, the FP32 inversion function from a 4-bit count lane, the threshold
 // lookup in shared memory and the comparison, the adaptation and window counters, and a warp

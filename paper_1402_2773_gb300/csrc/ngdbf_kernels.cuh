@@ -55,7 +55,7 @@
 // 18 wide multiplies alone take 19 (1.05 cycles each), the ALU pipe 18, so the step is near the
 // issue and pipe limits (issue 62-68 %, ALU 57-61 % busy).  Forming E_k for every symbol took 103
 // cycles a step.  100003 frames at 4.5 dB (8-bit samples): 30.6 -> 12.5 ms; 200000 frames at 3.5 dB,
-// where 3 % of the outputs are evaluated and A and A' run every iteration: 260 -> 192 ms.  With
+// where 3 % of the outputs are evaluated and A and A' run every iteration: 260 -> 193 ms.  With
 // few slots an iteration is latency: 3.5 us for one frame of the (3,6) code of 1008 symbols.
 //
 // The single-bit variant (Step 3a) needs the least E_k of a slot: it sweeps with a guess tau, the
@@ -262,7 +262,7 @@ __device__ __forceinline__ bool claim_frames(const Job& A, unsigned k, unsigned 
 // among 32, so launches that share the device pack their frames: twice as densely as those in flight and
 // the launch's own would lie over all CTAs, which leaves CTAs for launches to come, and comes to 32 a CTA
 // within a few generations of launches on a full device.  64 streams of 96 frames of the (6,32) code of
-// 2048 symbols at 3.0 dB, 256 calls: 62 ms packed by 32, 251 spread, 57 so; one such call by itself 1.4 ms
+// 2048 symbols at 3.0 dB, 256 calls: 62 ms packed by 32, 252 spread, 55 so; one such call by itself 1.4 ms
 // at 4.0 dB (7.3 packed).  (The launch's own frames in flight are at most those claimed from its queue, read
 // after the total: by itself it sees no others.)
 __device__ __forceinline__ unsigned busy_slots(const Job& A) {

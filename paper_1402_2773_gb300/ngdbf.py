@@ -324,7 +324,7 @@ def ngdbf_generator_table() -> np.ndarray:
 
 
 def ngdbf_mix_probe(groups: int, sink_ptr: int, stream: int = 0) -> int:
-    """Launches the same-mix throughput probe; returns the number of threads launched."""
+    """Launches the dense-mix throughput probe; returns the number of threads launched."""
     lib = load()
     th = ctypes.c_int64()
     _check(lib, lib.ngdbf_mix_probe(groups, sink_ptr, ctypes.byref(th), stream))
