@@ -744,7 +744,7 @@ struct PhiloxKeys {
     uint32_t rk0[10], rk1[10];
 };
 
-// Iterations with every E_k formed (narrow codes outside clusters, Step 3b, no trace), lane =
+// Iterations with every E_k formed (narrow codes outside clusters, adaptive variants, no trace), lane =
 // slot, for a CTA of more than 16 live slots of whose outputs so many are at or below their cutoffs
 // that the exact form of those one by one costs more.  Takes over after phase C of iteration `round`,
 // in which tally[0] outputs were evaluated; runs phases A, A' and C until a slot finishes or the flips
@@ -1398,7 +1398,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         // ---- A'. per symbol and slot, the count of unsatisfied checks in M(k) ----
         uint32_t* n_flips = ctl + 6 + (round & 1);
         if (tid == 0) ctl[6 + ((round + 1) & 1)] = 0u;
-        if (!WIDE && !CL && !single && tid == 0 && (round & kFullEvery) == kFullEvery - 1) tally[0] = 0u;
+        if (!WIDE && !CL && ADAPT && !single && tid == 0 && (round & kFullEvery) == kFullEvery - 1) tally[0] = 0u;
         if (anew) {
         // a CTA of a split job flips decisions in every copy during phase C: none before every
         // CTA has formed its syndromes (the barrier's wait is below, after the counts)
@@ -1627,7 +1627,7 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
             if (lg == 5) run(std::true_type{});
             else run(std::false_type{});
             while (queued) evaluate(queued < 32 ? queued : 32);
-            if (!CL && !single && (round & kFullEvery) == kFullEvery && lane == 0 && evaluated) atomicAdd(tally, (unsigned)evaluated);
+            if (!CL && ADAPT && !single && (round & kFullEvery) == kFullEvery && lane == 0 && evaluated) atomicAdd(tally, (unsigned)evaluated);
         } else {
             // every symbol of every slot, lane = slot (an idle slot's decisions and counters are
             // don't-care: cleared when it takes a frame, never part of an output)
@@ -1748,8 +1748,10 @@ __device__ __forceinline__ void decode_job(const Job& A, const uint32_t* thr_src
         anew = true;
         if constexpr (!WIDE) {
             // (not in cluster kernels, whose hot code it cost 4 % of the five-code workload: 1.446 -> 1.387 M
-            // frames/s; a table's shape is chosen by its measured time)
-            if constexpr (!CL) {
+            // frames/s; a table's shape is chosen by its measured time.  Not without adaptation: thresholds
+            // that do not rise leave few outputs to evaluate -- 20000 frames of the plain decoder at 0 dB take
+            // 4.2 ms lazy, 5.0 with every E_k formed -- and the call cost 72 frames of it 6 %)
+            if constexpr (!CL && ADAPT) {
                 if (!single && (round & kFullEvery) == kFullEvery && __popc(live) > kSlots / 2 &&
                     tally[0] > (uint32_t)(groups_l * kFullMarks) && A.trace_u == nullptr) {
                     round = full_rounds<ADAPT, SMOOTH, ST_SMEM, PREC, CHAIN>(

@@ -1,6 +1,6 @@
 """Batches so noisy that most outputs are at or below their cutoffs, vs the reference decoder, bit for
-bit: CTAs with more than half of their slots live go over from the lazy form to one that forms
-every E_k and back, with frames that finish, are refilled or run out on both sides of it.
+bit: in the adaptive variants CTAs with more than half of their slots live go over from the lazy
+form to one that forms every E_k and back, with frames that finish, are refilled or run out on both sides of it.
 """
 import numpy as np
 import pytest
